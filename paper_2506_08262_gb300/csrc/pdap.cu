@@ -1919,77 +1919,127 @@ int pdap_max_group(int n, int ldx, int m, int d, bool keys_in, bool allow_stream
 // Keys of a block of tasks (G directions each, all of one dataset) for every point, as a tiled FP32
 // GEMM: keys[(t * G + g) * npad + i] = u_{t,g}'x_i, each key one sequential FMA chain over the dims
 // (the selection kernel's own arithmetic for d > 16, and y_z's), so results do not depend on which
-// kernel formed the keys.  CTA tile: 128 points x 128 directions, 256 threads of 8 x 8 outputs, the
-// dims staged 16 at a time in shared memory.
-constexpr int KT_P = 128, KT_D = 128, KT_K = 16;
+// kernel formed the keys.
+//
+// Bound by the FMA pipe and the register ports in front of it.  CTA tile 128 points x 128 directions, 128
+// threads, two CTAs per SM; a thread takes 16 points x 8 directions as 8 point pairs x 8 directions, each
+// pair one packed FMA (fma.rn.f32x2: two IEEE FMAs, so every key keeps its chain, in one issue slot).  Per
+// dim a thread issues 64 packed FMAs on 6 shared loads; lanes read 16-byte words that are consecutive over
+// the 8 point lanes and the 4 direction lanes of a warp, so no load has a bank conflict.  The dims come 16 at
+// a time, the next 16 in flight in registers during the FMAs, two staging buffers, one barrier per step; the
+// last step runs only the dims that are there (rows are zero-padded to a multiple of 4).
+// Measured, 10,000 points x 6,700 directions: d = 50 243 -> 164 us, d = 100 295 us (56% of the FMA peak).
+// 8 x 8 outputs per thread, directions duplicated in shared memory: 204 us (shared-memory loads 68% busy);
+// duplicated in registers: 181 us; scalar FMAs: 181 us; row-major staging by cp.async: 168 us at best.
+constexpr int KT_P = 128, KT_D = 128, KT_K = 16, KT_NT = 128;
 
-__global__ void __launch_bounds__(256) k_keys(const TaskDev* __restrict__ tasks, int ntasks, int G,
-                                              const SlotDev* __restrict__ slots, const DsDev* __restrict__ dsets,
-                                              const float* __restrict__ U, float* __restrict__ keys, int npad)
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
 {
-    __shared__ __align__(16) float Xs[KT_K][KT_P + 4];   // [dim][point]
-    __shared__ __align__(16) float Us[KT_K][KT_D + 4];   // [dim][direction]
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long dup2(float v)
+{
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(v));
+    return d;
+}
+
+__global__ void __launch_bounds__(KT_NT, 2) k_keys(const TaskDev* __restrict__ tasks, int ntasks, int G,
+                                                   const SlotDev* __restrict__ slots, const DsDev* __restrict__ dsets,
+                                                   const float* __restrict__ U, float* __restrict__ keys, int npad)
+{
+    __shared__ __align__(16) float Xs[2][KT_K][KT_P];   // [dim][point]
+    __shared__ __align__(16) float Us[2][KT_K][KT_D];   // [dim][direction]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const DsDev D = dsets[slots[tasks[0].slot].ds];
     const int n = (int)D.n, ldx = D.ldx, dp4 = (D.d + 3) & ~3;
     const int i0 = blockIdx.x * KT_P, r0 = blockIdx.y * KT_D;
-    // staging: thread tid loads 8 dims of point row tid / 2 and 8 dims of direction row tid / 2
-    const int lr = tid >> 1, lh = (tid & 1) * 8;
+    // staging: thread tid loads the 16 dims of point row tid and of direction row tid (a warp's 32 rows are
+    // consecutive, so its transposed stores are free of conflicts)
     const float* urow = nullptr;
     {
-        const int r = r0 + lr, t = r / G, g = r - t * G;
+        const int r = r0 + tid, t = r / G, g = r - t * G;
         if (t < ntasks && g < tasks[t].nj) {
             const TaskDev T = tasks[t];
             urow = U + slots[T.slot].uoff + (int64_t)(T.j0 + g) * ldx;
         }
     }
-    const float* xrow = (i0 + lr < n) ? D.X32 + (int64_t)(i0 + lr) * ldx : nullptr;
-    float acc[8][8];
+    const float* xrow = (i0 + tid < n) ? D.X32 + (int64_t)(i0 + tid) * ldx : nullptr;
+    float4 xg[KT_K / 4], ug[KT_K / 4];   // the next step's dims
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int h = 0; h < KT_K / 4; ++h) {
+            const int l = k0 + 4 * h;
+            xg[h] = ug[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (xrow && l < dp4) xg[h] = *reinterpret_cast<const float4*>(xrow + l);
+            if (urow && l < dp4) ug[h] = *reinterpret_cast<const float4*>(urow + l);
+        }
+    };
+    auto stage = [&](int b) {
+#pragma unroll
+        for (int h = 0; h < KT_K / 4; ++h) {
+            const float xv[4] = {xg[h].x, xg[h].y, xg[h].z, xg[h].w}, uv[4] = {ug[h].x, ug[h].y, ug[h].z, ug[h].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                Xs[b][4 * h + e][tid] = xv[e];
+                Us[b][4 * h + e][tid] = uv[e];
+            }
+        }
+    };
+    // this thread's points p0 + 32 a + {0..3}, a = 0..3, and directions q0 + 16 c + {0..3}, c = 0, 1
+    const int p0 = (lane & 7) * 4, q0 = warp * 32 + (lane >> 3) * 4;
+    unsigned long long acc[8][8];   // [point pair][direction]
 #pragma unroll
     for (int a = 0; a < 8; ++a)
 #pragma unroll
-        for (int b = 0; b < 8; ++b) acc[a][b] = 0.0f;
-    for (int k0 = 0; k0 < dp4; k0 += KT_K) {
-        // zero beyond the row (rows are zero-padded to ldx, so the extra terms add exact zeros)
+        for (int c = 0; c < 8; ++c) acc[a][c] = 0ull;
+    fetch(0);
+    stage(0);
+    __syncthreads();
+    int b = 0;
+    for (int k0 = 0; k0 < dp4; k0 += KT_K, b ^= 1) {
+        const bool more = k0 + KT_K < dp4;
+        if (more) fetch(k0 + KT_K);
+        const int kc = dp4 - k0 < KT_K ? dp4 - k0 : KT_K;
+        for (int k4 = 0; k4 < kc; k4 += 4) {
 #pragma unroll
-        for (int h = 0; h < 8; h += 4) {
-            const int l = k0 + lh + h;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f), w = v;
-            if (xrow && l + 4 <= ldx) v = *reinterpret_cast<const float4*>(xrow + l);
-            if (urow && l + 4 <= ldx) w = *reinterpret_cast<const float4*>(urow + l);
-            Xs[lh + h][lr] = v.x;
-            Xs[lh + h + 1][lr] = v.y;
-            Xs[lh + h + 2][lr] = v.z;
-            Xs[lh + h + 3][lr] = v.w;
-            Us[lh + h][lr] = w.x;
-            Us[lh + h + 1][lr] = w.y;
-            Us[lh + h + 2][lr] = w.z;
-            Us[lh + h + 3][lr] = w.w;
+            for (int e = 0; e < 4; ++e) {
+                const float* xs = &Xs[b][k4 + e][p0];
+                unsigned long long xv[8];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    const ulonglong2 x2 = *reinterpret_cast<const ulonglong2*>(xs + 32 * a);
+                    xv[2 * a] = x2.x;
+                    xv[2 * a + 1] = x2.y;
+                }
+                const float* us = &Us[b][k4 + e][q0];
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const float4 u4 = *reinterpret_cast<const float4*>(us + 16 * c);
+                    const float uv[4] = {u4.x, u4.y, u4.z, u4.w};
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const unsigned long long ud = dup2(uv[h]);
+#pragma unroll
+                        for (int a = 0; a < 8; ++a) acc[a][4 * c + h] = fma2(ud, xv[a], acc[a][4 * c + h]);
+                    }
+                }
+            }
         }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < KT_K; ++kk) {
-            const float4 a0 = *reinterpret_cast<const float4*>(&Xs[kk][tx * 8]);
-            const float4 a1 = *reinterpret_cast<const float4*>(&Xs[kk][tx * 8 + 4]);
-            const float4 b0 = *reinterpret_cast<const float4*>(&Us[kk][ty * 8]);
-            const float4 b1 = *reinterpret_cast<const float4*>(&Us[kk][ty * 8 + 4]);
-            const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-            for (int a = 0; a < 8; ++a)
-#pragma unroll
-                for (int c = 0; c < 8; ++c) acc[a][c] = fmaf(bv[c], av[a], acc[a][c]);
-        }
+        if (more) stage(b ^ 1);   // the buffer whose readers passed the last barrier
         __syncthreads();
     }
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-        const int r = r0 + ty * 8 + c, t = r / G, g = r - t * G;
+        const int r = r0 + q0 + 16 * (c >> 2) + (c & 3), t = r / G, g = r - t * G;
         if (t >= ntasks || g >= tasks[t].nj) continue;
-        float* out = keys + (size_t)r * npad + i0 + tx * 8;
-        if (i0 + tx * 8 + 4 <= npad) *reinterpret_cast<float4*>(out) = make_float4(acc[0][c], acc[1][c], acc[2][c], acc[3][c]);
-        if (i0 + tx * 8 + 8 <= npad)
-            *reinterpret_cast<float4*>(out + 4) = make_float4(acc[4][c], acc[5][c], acc[6][c], acc[7][c]);
+        float* out = keys + (size_t)r * npad + i0 + p0;
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            if (i0 + p0 + 32 * a + 4 <= npad)
+                *reinterpret_cast<ulonglong2*>(out + 32 * a) = make_ulonglong2(acc[2 * a][c], acc[2 * a + 1][c]);
     }
 }
 
@@ -2208,7 +2258,7 @@ cudaError_t launch_pdap_keys(const TaskDev* tasks, int ntasks, int group, const 
         return cudaGetLastError();
     }
     const dim3 grid((unsigned)((ds_host.n + KT_P - 1) / KT_P), (unsigned)((ntasks * group + KT_D - 1) / KT_D));
-    k_keys<<<grid, 256, 0, st>>>(tasks, ntasks, group, slots, ds, U, keys, npad);
+    k_keys<<<grid, KT_NT, 0, st>>>(tasks, ntasks, group, slots, ds, U, keys, npad);
     return cudaGetLastError();
 }
 
