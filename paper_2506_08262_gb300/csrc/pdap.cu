@@ -28,6 +28,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "packed_fma.cuh"
 #include "rrs_internal.h"
 
 namespace rrs {
@@ -1932,19 +1933,6 @@ int pdap_max_group(int n, int ldx, int m, int d, bool keys_in, bool allow_stream
 // 8 x 8 outputs per thread, directions duplicated in shared memory: 204 us (shared-memory loads 68% busy);
 // duplicated in registers: 181 us; scalar FMAs: 181 us; row-major staging by cp.async: 168 us at best.
 constexpr int KT_P = 128, KT_D = 128, KT_K = 16, KT_NT = 128;
-
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c)
-{
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ unsigned long long dup2(float v)
-{
-    unsigned long long d;
-    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(v));
-    return d;
-}
 
 __global__ void __launch_bounds__(KT_NT, 2) k_keys(const TaskDev* __restrict__ tasks, int ntasks, int G,
                                                    const SlotDev* __restrict__ slots, const DsDev* __restrict__ dsets,

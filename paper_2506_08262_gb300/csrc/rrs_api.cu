@@ -150,6 +150,7 @@ struct Plan {
     std::vector<std::vector<int>> n_pd;
     int rmax = 0;
     int max_ldx = 4;
+    int64_t hd_n = 0;   // largest n among the FP32 halfspace datasets
     int64_t tot_ldx = 0, tot_d = 0, tot_u = 0, tot_m = 0;
     // tensor-core halfspace tasks, one group per K extent of the planes (64 or 128), each group one launch
     // per round whatever the datasets: every task's CTA takes its dataset's tensor map from maps
@@ -322,17 +323,18 @@ rrs_status build_plan(const std::vector<ReqView>& reqs, Plan& P)
             P.tot_d += D.d;
             P.max_ldx = std::max(P.max_ldx, D.ldx);
             for (int j0 = 0; j0 < m; j0 += 128) P.gen_tasks.push_back(TaskDev{s, j0, std::min(128, m - j0), 0});
-            if (R.kind == RRS_HALFSPACE) {
-                if (!tc) {
-                    const int cap = 64;   // directions per CTA of the FP32 kernel
-                    const int nt = (m + cap - 1) / cap;
-                    const int per = (m + nt - 1) / nt;
-                    for (int j0 = 0; j0 < m; j0 += per) P.hd_tasks.push_back(TaskDev{s, j0, std::min(per, m - j0), 0});
-                }
-            } else {
+            if (R.kind != RRS_HALFSPACE) {
                 for (int j0 = 0; j0 < m; j0 += G) P.pd_tasks[cls].push_back(TaskDev{s, j0, std::min(G, m - j0), S.ds});
             }
             P.argmin_list.push_back(s);
+        }
+        if (R.kind == RRS_HALFSPACE && !tc) {
+            // FP32 tasks: HD_ROWS consecutive (query, direction) rows of this request, across its queries
+            const int64_t rows = R.nq * (int64_t)m;
+            P.hd_n = std::max(P.hd_n, D.n);
+            for (int64_t g = 0; g < rows; g += HD_ROWS)
+                P.hd_tasks.push_back(
+                    TaskDev{s_first + (int)(g / m), (int)(g % m), (int)std::min<int64_t>(HD_ROWS, rows - g), 0});
         }
         if (tc) {
             // tensor-core tasks: 128 consecutive (query, direction) rows of this request, so the
@@ -457,13 +459,13 @@ rrs_status enqueue_rounds(rrs_ctx* ctx, Plan& P, cudaStream_t st, bool capturing
         float* nxt = P.poles + ((l + 1) & 1) * T;
         if (P.n_gen[l] > 0) {
             StageTimer t(ctx, RRS_STAGE_GEN, st, capturing);
-            CUDA_TRY(launch_gen(P.d_gen, P.n_gen[l], P.d_slots, cur, P.z64, P.U, P.yz, l, P.max_ldx, st));
+            CUDA_TRY(launch_gen(P.d_gen, P.n_gen[l], P.d_slots, cur, P.z64, P.U, P.yz, P.res, l, P.max_ldx, st));
             ctx->launches++;
             ctx->stage_launches[RRS_STAGE_GEN]++;
         }
         if (P.n_hd[l] > 0) {
             StageTimer t(ctx, RRS_STAGE_HD_SIMT, st, capturing);
-            CUDA_TRY(launch_hd_simt(P.d_hd, P.n_hd[l], P.max_ldx, P.d_slots, P.d_ds, P.U, P.yz, P.z64, P.res,
+            CUDA_TRY(launch_hd_simt(P.d_hd, P.n_hd[l], P.max_ldx, P.hd_n, P.d_slots, P.d_ds, P.U, P.yz, P.z64, P.res,
                                     nullptr, ctx->d_err, st));
             ctx->stage_launches[RRS_STAGE_HD_SIMT]++;
             ctx->launches++;
@@ -1013,7 +1015,7 @@ rrs_status rrs_debug_round_depths(rrs_ctx* ctx, int64_t dataset_id, const void* 
                 CUDA_TRY(launch_hd_tc(P.tc[0].d, (int)P.tc[0].tasks.size(), P.tc[0].kp, P.tc[0].bn, P.d_slots, P.d_ds, P.d_maps, P.U, P.yz,
                                       P.z64, P.res, band, ctx->d_err, st));
             else
-                CUDA_TRY(launch_hd_simt(P.d_hd, (int)P.hd_tasks.size(), P.max_ldx, P.d_slots, P.d_ds, P.U, P.yz,
+                CUDA_TRY(launch_hd_simt(P.d_hd, (int)P.hd_tasks.size(), P.max_ldx, 0, P.d_slots, P.d_ds, P.U, P.yz,
                                         P.z64, P.res, band, ctx->d_err, st));
         } else {
             for (size_t c = 0; c < P.pd_tasks.size(); ++c)

@@ -7,6 +7,9 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
+#include "packed_fma.cuh"
 #include "rrs_device.cuh"
 #include "rrs_internal.h"
 
@@ -210,7 +213,7 @@ constexpr size_t GEN_STAGE_MAX = 96 * 1024;
 __global__ void __launch_bounds__(GEN_NT) k_gen(const TaskDev* __restrict__ tasks, const SlotDev* __restrict__ slots,
                                                 const float* __restrict__ poles, const float* __restrict__ poles1,
                                                 const double* __restrict__ z64, float* __restrict__ U,
-                                                double* __restrict__ yz, int round0, int stage_d)
+                                                double* __restrict__ yz, ResDev* __restrict__ res, int round0, int stage_d)
 {
     extern __shared__ float gstage[];
     const TaskDev T = tasks[blockIdx.x];
@@ -222,6 +225,8 @@ __global__ void __launch_bounds__(GEN_NT) k_gen(const TaskDev* __restrict__ task
     const int j = T.j0 + jl;
     const float ap = alpha_power(S.alpha, rnd);
     const double* z = z64 + S.zoff64;
+    // zero result cells: where the halfspace kernel splits the points it adds its counts there
+    if (jl < T.nj) res[S.roff + j] = ResDev{0.0, 0};
     if (S.d > stage_d) {
         if (jl >= T.nj) return;
         float* u = U + S.uoff + (int64_t)j * S.ldx;
@@ -252,8 +257,8 @@ __global__ void __launch_bounds__(GEN_NT) k_gen(const TaskDev* __restrict__ task
 
 // directions of up to max_ldx dims are staged in shared memory (up to GEN_STAGE_MAX bytes)
 static cudaError_t gen_launch(const TaskDev* tasks, int ntasks, const SlotDev* slots, const float* p0,
-                              const float* p1, const double* z64, float* U, double* yz, int round0, int max_ldx,
-                              cudaStream_t st)
+                              const float* p1, const double* z64, float* U, double* yz, ResDev* res, int round0,
+                              int max_ldx, cudaStream_t st)
 {
     if (ntasks <= 0) return cudaSuccess;
     int stage_d = max_ldx;
@@ -267,21 +272,21 @@ static cudaError_t gen_launch(const TaskDev* tasks, int ntasks, const SlotDev* s
             return e;
         }
     }
-    k_gen<<<ntasks, GEN_NT, smem, st>>>(tasks, slots, p0, p1, z64, U, yz, round0, stage_d);
+    k_gen<<<ntasks, GEN_NT, smem, st>>>(tasks, slots, p0, p1, z64, U, yz, res, round0, stage_d);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gen(const TaskDev* tasks, int ntasks, const SlotDev* slots, const float* poles_cur,
-                       const double* z64, float* U, double* yz, int round0, int max_ldx, cudaStream_t st)
+                       const double* z64, float* U, double* yz, ResDev* res, int round0, int max_ldx, cudaStream_t st)
 {
-    return gen_launch(tasks, ntasks, slots, poles_cur, nullptr, z64, U, yz, round0, max_ldx, st);
+    return gen_launch(tasks, ntasks, slots, poles_cur, nullptr, z64, U, yz, res, round0, max_ldx, st);
 }
 
 cudaError_t launch_gen_slotround(const TaskDev* tasks, int ntasks, const SlotDev* slots, const float* poles0,
-                                 const float* poles1, const double* z64, float* U, double* yz, int max_ldx,
-                                 cudaStream_t st)
+                                 const float* poles1, const double* z64, float* U, double* yz, ResDev* res,
+                                 int max_ldx, cudaStream_t st)
 {
-    return gen_launch(tasks, ntasks, slots, poles0, poles1, z64, U, yz, -1, max_ldx, st);
+    return gen_launch(tasks, ntasks, slots, poles0, poles1, z64, U, yz, res, -1, max_ldx, st);
 }
 
 // y_z = u'z in FP64 for caller-supplied directions (debug path)
@@ -350,142 +355,296 @@ cudaError_t launch_debug_dirs(uint64_t seed, int q, int round0, int m, int d, fl
 // halfspace counts, FP32 SIMT projection + exact recheck of the near-tie band
 // ---------------------------------------------------------------------------
 
-constexpr int HD_NT = 256;
-constexpr int HD_TJ = 64;   // directions per CTA
-constexpr int HD_PC = 64;   // points per staged chunk
+// One CTA takes up to HD_TJ consecutive (query, direction) rows of one request and walks the points in chunks of
+// HD_PC.  Bound by the FMA pipe and the register ports in front of it; the projection is k_keys' register tile
+// (16 points x 8 directions per thread as packed FMAs, fma2 / dup2).  Each accumulator starts at -u'z, so the chain
+// ends in t = u'x - u'z itself, and the comparison with the band costs three slots per pair: packed t + b and
+// b - t, whose sign bits (t < -b, t > b) are shifted into one word per direction and counted.  Pairs with neither
+// bit set are near ties and take the exact test.  The directions stay in shared memory; the points come 16 dims at
+// a time, the next 16 in flight in registers.
+// Measured at d = 50, n = 100,000, 100 queries of 100 directions: 9.28 ms per round with 4 x 4 scalar outputs per
+// thread, 5.11 ms with this tile, 2.78 ms with the points also split (hd_parts): 46% of the FMA peak.
+constexpr int HD_NT = 128;
+constexpr int HD_TJ = HD_ROWS;   // rows (query, direction) per CTA
+constexpr int HD_PC = 256;       // points per chunk
+constexpr int HD_K = 16;         // dims per staging step
+constexpr int HD_PART_SHIFT = 48;   // bits of a count in a result cell shared by the parts of a split (n < 2^48)
 
-__global__ void __launch_bounds__(HD_NT) k_hd_simt(const TaskDev* __restrict__ tasks,
-                                                   const SlotDev* __restrict__ slots, const DsDev* __restrict__ dsets,
-                                                   const float* __restrict__ U, const double* __restrict__ yz,
-                                                   const double* __restrict__ z64, ResDev* __restrict__ res,
-                                                   int64_t* __restrict__ band_out, int* err)
+// Parts the points are split into.  Two CTAs share an SM, and a launch of few tasks leaves SMs empty or ends in a
+// wave that is nearly empty: below eight waves of tasks the points are split into as many parts as give about
+// eight waves, each of at least HD_MIN_CHUNKS chunks (a part stages its directions again and meets the others in
+// the result cells).  Measured, 157 tasks at d = 50, n = 100,000: 5.11 ms per round unsplit, 2.78 ms in 16 parts.
+constexpr int HD_WAVE = 2 * 152, HD_MIN_CHUNKS = 4;
+static int hd_parts(int ntasks, int64_t max_n)
+{
+    if (ntasks >= 8 * HD_WAVE) return 1;
+    const int64_t chunks = (max_n + HD_PC - 1) / HD_PC, want = (8 * HD_WAVE + ntasks - 1) / ntasks;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(want, chunks / HD_MIN_CHUNKS));
+}
+
+// Exact sign of u'(x_i - z) of one near tie; a call of its own, so the register tile's code stays small.
+__device__ __noinline__ int hd_exact(const DsDev& D, const float* u, int64_t i, const double* z, int* err)
+{
+    if (D.X64) return exact_sign<double>(u, 1, D.X64 + i * D.d, z, D.d, err);
+    return exact_sign<float>(u, 1, D.X32 + i * D.ldx, z, D.d, err);
+}
+
+__global__ void __launch_bounds__(HD_NT, 2) k_hd_simt(const TaskDev* __restrict__ tasks,
+                                                      const SlotDev* __restrict__ slots,
+                                                      const DsDev* __restrict__ dsets, const float* __restrict__ U,
+                                                      const double* __restrict__ yz, const double* __restrict__ z64,
+                                                      ResDev* __restrict__ res, int64_t* __restrict__ band_out, int* err)
 {
     extern __shared__ __align__(16) float sm[];
+    __shared__ int64_t r_uoff[HD_TJ], r_zoff[HD_TJ], r_roff[HD_TJ];
+    __shared__ int r_slot[HD_TJ];
+    __shared__ unsigned long long c_lt[HD_TJ], c_gt[HD_TJ];
+    __shared__ float r_ny[HD_TJ];
+    __shared__ unsigned zmax_bits;
     const TaskDev T = tasks[blockIdx.x];
-    const SlotDev& S = slots[T.slot];
-    const DsDev D = dsets[S.ds];
+    const DsDev D = dsets[slots[T.slot].ds];
     const int ldx = D.ldx, d = D.d, dp4 = (d + 3) & ~3;
     const int64_t n = D.n;
-    float* uS = sm;                       // HD_TJ x ldx
-    float* xS = uS + HD_TJ * ldx;         // HD_PC x ldx
-    float* xnS = xS + HD_PC * ldx;        // HD_PC
-    float* yzS = xnS + HD_PC;             // HD_TJ
-    const int tid = threadIdx.x;
+    float* Xs = sm;                              // 2 x HD_K x HD_PC: [dim][point]
+    float* bS = Xs + 2 * HD_K * HD_PC;           // 2 x HD_PC: band bound of each point of the chunk
+    float* Us = bS + 2 * HD_PC;                  // dp4 x HD_TJ: [dim][row]
+    // this CTA's points: part blockIdx.y of nparts, in whole chunks
+    const int64_t nch = (n + HD_PC - 1) / HD_PC, per = (nch + gridDim.y - 1) / gridDim.y;
+    const int nparts = (int)((nch + per - 1) / per);
+    const int64_t ibeg = (int64_t)blockIdx.y * per * HD_PC;
+    if (ibeg >= n) return;
+    const int64_t iend = ibeg + per * HD_PC < n ? ibeg + per * HD_PC : n;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    for (int e = tid; e < HD_TJ * ldx; e += HD_NT) {
-        const int j = e / ldx;
-        uS[e] = (j < T.nj) ? U[S.uoff + (int64_t)(T.j0 + j) * ldx + (e - j * ldx)] : 0.0f;
-    }
-    for (int j = tid; j < HD_TJ; j += HD_NT) yzS[j] = (j < T.nj) ? (float)yz[S.roff + T.j0 + j] : 0.0f;
-
-    const float gamma = band_gamma_fp32(d);
-    const float zn = S.znorm;
-    const double* zrow = z64 + S.zoff64;
-    const int dg = tid >> 4, pg = tid & 15;
-    int lt[4] = {0, 0, 0, 0}, gt[4] = {0, 0, 0, 0};
-    int nband = 0;
-
-    for (int64_t i0 = 0; i0 < n; i0 += HD_PC) {
-        __syncthreads();
-        const int64_t rows = (n - i0 < HD_PC) ? (n - i0) : HD_PC;
-        const float4* src = reinterpret_cast<const float4*>(D.X32 + i0 * ldx);
-        float4* dst = reinterpret_cast<float4*>(xS);
-        const int nv = HD_PC * ldx / 4, nvalid = (int)rows * ldx / 4;
-        for (int e = tid; e < nv; e += HD_NT) dst[e] = (e < nvalid) ? src[e] : make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int p = tid; p < HD_PC; p += HD_NT) xnS[p] = (p < rows) ? D.xnorm[i0 + p] : 0.0f;
-        __syncthreads();
-
-        float acc[4][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int t = 0; t < 4; ++t) acc[a][t] = 0.0f;
-        for (int l = 0; l < dp4; l += 4) {
-            float4 uv[4], xv[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) uv[a] = *reinterpret_cast<const float4*>(uS + (dg * 4 + a) * ldx + l);
-#pragma unroll
-            for (int t = 0; t < 4; ++t) xv[t] = *reinterpret_cast<const float4*>(xS + (pg + 16 * t) * ldx + l);
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    acc[a][t] = fmaf(uv[a].x, xv[t].x, acc[a][t]);
-                    acc[a][t] = fmaf(uv[a].y, xv[t].y, acc[a][t]);
-                    acc[a][t] = fmaf(uv[a].z, xv[t].z, acc[a][t]);
-                    acc[a][t] = fmaf(uv[a].w, xv[t].w, acc[a][t]);
-                }
+    if (tid == 0) zmax_bits = 0u;
+    __syncthreads();
+    if (tid < HD_TJ) {
+        const int r = tid;
+        c_lt[r] = c_gt[r] = 0ull;
+        r_ny[r] = 0.0f;
+        r_slot[r] = -1;
+        if (r < T.nj) {
+            const int m = slots[T.slot].m;
+            const int gg = T.j0 + r, qs = gg / m, j = gg - qs * m;   // rows may run into the request's next queries
+            const SlotDev& S = slots[T.slot + qs];
+            r_slot[r] = T.slot + qs;
+            r_uoff[r] = S.uoff + (int64_t)j * ldx;
+            r_zoff[r] = S.zoff64;
+            r_roff[r] = S.roff + j;
+            r_ny[r] = -(float)yz[S.roff + j];
+            atomicMax(&zmax_bits, __float_as_uint(S.znorm));   // norms are not negative
         }
+    }
+    __syncthreads();
+    for (int e = tid; e < HD_TJ * (dp4 / 4); e += HD_NT) {
+        const int r = e & (HD_TJ - 1), l = (e / HD_TJ) * 4;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < T.nj) v = *reinterpret_cast<const float4*>(U + r_uoff[r] + l);
+        Us[l * HD_TJ + r] = v.x;
+        Us[(l + 1) * HD_TJ + r] = v.y;
+        Us[(l + 2) * HD_TJ + r] = v.z;
+        Us[(l + 3) * HD_TJ + r] = v.w;
+    }
+    const float gamma = band_gamma_fp32(d), gz = gamma * __uint_as_float(zmax_bits);
+
+    // staging: thread tid takes point rows tid and tid + 128 of the chunk (transposed stores free of conflicts)
+    float4 xg[2][HD_K / 4];
+    float xn[2];
+    auto fetch = [&](int64_t i0, int k0) {
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int p = pg + 16 * t;
-            if (p >= rows) continue;
-            const float b = gamma * (xnS[p] + zn);
+        for (int p = 0; p < 2; ++p) {
+            const int64_t i = i0 + tid + p * HD_NT;
+            const float* xr = D.X32 + i * ldx + k0;
+            if (k0 == 0) xn[p] = i < n ? D.xnorm[i] : 0.0f;
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const int j = dg * 4 + a;
-                if (j >= T.nj) continue;
-                const float tv = acc[a][t] - yzS[j];
-                if (tv < -b) {
-                    lt[a]++;
-                } else if (tv > b) {
-                    gt[a]++;
-                } else {
-                    const int64_t i = i0 + p;
-                    int s;
-                    if (D.X64) s = exact_sign<double>(uS + j * ldx, 1, D.X64 + i * d, zrow, d, err);
-                    else s = exact_sign<float>(uS + j * ldx, 1, D.X32 + i * ldx, zrow, d, err);
-                    lt[a] += (s < 0);
-                    gt[a] += (s > 0);
-                    nband++;
+            for (int h = 0; h < HD_K / 4; ++h) {
+                xg[p][h] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (i < n && k0 + 4 * h < dp4) xg[p][h] = *reinterpret_cast<const float4*>(xr + 4 * h);
+            }
+        }
+    };
+    auto stage = [&](int b, int cb, bool first) {
+        float* xs = Xs + b * HD_K * HD_PC + tid;
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            if (first) bS[cb * HD_PC + tid + p * HD_NT] = fmaf(gamma, xn[p], gz);
+#pragma unroll
+            for (int h = 0; h < HD_K / 4; ++h) {
+                xs[(4 * h) * HD_PC + p * HD_NT] = xg[p][h].x;
+                xs[(4 * h + 1) * HD_PC + p * HD_NT] = xg[p][h].y;
+                xs[(4 * h + 2) * HD_PC + p * HD_NT] = xg[p][h].z;
+                xs[(4 * h + 3) * HD_PC + p * HD_NT] = xg[p][h].w;
+            }
+        }
+    };
+    // this thread's points p0 + 32 a + {0..3}, a = 0..3, and rows q0 + 16 c + {0..3}, c = 0, 1
+    const int p0 = (warp & 1) * 128 + (lane & 7) * 4, q0 = (warp >> 1) * 32 + (lane >> 3) * 4;
+    auto row_of = [&](int c) { return q0 + 16 * (c >> 2) + (c & 3); };
+    unsigned long long acc[8][8];   // [point pair][row]
+    auto reset = [&] {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const unsigned long long y = dup2(r_ny[row_of(c)]);
+#pragma unroll
+            for (int a = 0; a < 8; ++a) acc[a][c] = y;
+        }
+    };
+    int lt[8], gt[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) lt[c] = gt[c] = 0;
+
+    fetch(ibeg, 0);
+    stage(0, 0, true);
+    __syncthreads();
+    reset();
+    int64_t i0 = ibeg;
+    int k0 = 0, b = 0, cb = 0;
+    for (;;) {
+        int64_t ni = i0;
+        int nk = k0 + HD_K;
+        if (nk >= dp4) {
+            nk = 0;
+            ni = i0 + HD_PC;
+        }
+        const bool last_k = nk == 0, more = ni < iend;
+        if (more) fetch(ni, nk);
+        const int kc = dp4 - k0 < HD_K ? dp4 - k0 : HD_K;
+        for (int k4 = 0; k4 < kc; k4 += 4) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float* xs = Xs + (b * HD_K + k4 + e) * HD_PC + p0;
+                unsigned long long xv[8];
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    const ulonglong2 x2 = *reinterpret_cast<const ulonglong2*>(xs + 32 * a);
+                    xv[2 * a] = x2.x;
+                    xv[2 * a + 1] = x2.y;
+                }
+                const float* us = Us + (k0 + k4 + e) * HD_TJ + q0;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const float4 u4 = *reinterpret_cast<const float4*>(us + 16 * c);
+                    const float uv[4] = {u4.x, u4.y, u4.z, u4.w};
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const unsigned long long ud = dup2(uv[h]);
+#pragma unroll
+                        for (int a = 0; a < 8; ++a) acc[a][4 * c + h] = fma2(ud, xv[a], acc[a][4 * c + h]);
+                    }
                 }
             }
         }
-    }
+        if (last_k) {
+            // bits 31 - k and 15 - k of w[c]: t < -b and t > b of the thread's k-th point, row c
+            unsigned w[8];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
+            for (int c = 0; c < 8; ++c) w[c] = 0u;
+            const float* bp = bS + cb * HD_PC + p0;
 #pragma unroll
-        for (int o = 8; o >= 1; o >>= 1) {
-            lt[a] += __shfl_xor_sync(0xFFFFFFFFu, lt[a], o);
-            gt[a] += __shfl_xor_sync(0xFFFFFFFFu, gt[a], o);
-        }
-    }
-    if (band_out) {
-        // band points are counted per thread over its directions; one total per CTA task
-        __shared__ int bsum;
-        if (tid == 0) bsum = 0;
-        __syncthreads();
-        atomicAdd(&bsum, nband);
-        __syncthreads();
-        if (tid == 0) atomicAdd((unsigned long long*)&band_out[T.slot], (unsigned long long)bsum);
-    }
-    if (pg == 0) {
+            for (int pass = 0; pass < 2; ++pass) {
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const int j = dg * 4 + a;
-            if (j < T.nj) {
-                const int64_t le = n - gt[a], ge = n - lt[a];
-                const int64_t c = le < ge ? le : ge;
-                res[S.roff + T.j0 + j] = ResDev{(double)c / (double)n, c};
+                for (int a = 0; a < 4; ++a) {
+                    const ulonglong2 b2 = *reinterpret_cast<const ulonglong2*>(bp + 32 * a);
+                    const unsigned long long bv[2] = {b2.x, b2.y};
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            // pass 0: b + t, negative where t < -b; pass 1: b - t, negative where t > b
+                            const unsigned long long s =
+                                pass == 0 ? add2(bv[h], acc[2 * a + h][c])
+                                          : fma2(acc[2 * a + h][c], 0xBF800000BF800000ull, bv[h]);
+                            w[c] = __funnelshift_l((unsigned)s, w[c], 1);
+                            w[c] = __funnelshift_l((unsigned)(s >> 32), w[c], 1);
+                        }
+                }
             }
+            // points of this thread that exist, first point in bit 15
+            unsigned vm = 0xFFFFu;
+            if (i0 + HD_PC > n) {
+                vm = 0u;
+#pragma unroll
+                for (int k = 0; k < 16; ++k) vm |= (unsigned)(i0 + p0 + 32 * (k >> 2) + (k & 3) < n) << (15 - k);
+            }
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const unsigned l = (w[c] >> 16) & vm, g = w[c] & vm;
+                lt[c] += __popc(l);
+                gt[c] += __popc(g);
+                unsigned cand = vm & ~(l | g);
+                const int r = row_of(c);
+                if (r >= T.nj) cand = 0u;
+                while (cand) {
+                    const int k = 31 - __clz(cand);
+                    cand &= ~(1u << k);
+                    const int pk = 15 - k;
+                    const int sgn = hd_exact(D, U + r_uoff[r], i0 + p0 + 32 * (pk >> 2) + (pk & 3),
+                                             z64 + r_zoff[r], err);
+                    lt[c] += sgn < 0;
+                    gt[c] += sgn > 0;
+                    if (band_out) atomicAdd((unsigned long long*)&band_out[r_slot[r]], 1ull);
+                }
+            }
+            if (more) reset();
+            cb ^= 1;
         }
+        if (!more) break;
+        stage(b ^ 1, cb, nk == 0);   // the buffer whose readers passed the last barrier
+        __syncthreads();
+        b ^= 1;
+        i0 = ni;
+        k0 = nk;
+    }
+    // the eight point lanes of a direction hold parts of its counts, and so do the two point warps
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        unsigned long long l = (unsigned)lt[c], g = (unsigned)gt[c];
+#pragma unroll
+        for (int o = 4; o >= 1; o >>= 1) {
+            l += __shfl_xor_sync(0xFFFFFFFFu, l, o);
+            g += __shfl_xor_sync(0xFFFFFFFFu, g, o);
+        }
+        if ((lane & 7) == 0) {
+            atomicAdd(&c_lt[row_of(c)], l);
+            atomicAdd(&c_gt[row_of(c)], g);
+        }
+    }
+    __syncthreads();
+    if (tid < T.nj) {
+        long long l = (long long)c_lt[tid], g = (long long)c_gt[tid];
+        ResDev* cell = res + r_roff[tid];
+        if (nparts > 1) {
+            // counts of the parts meet in the result cell (zeroed with the directions): #(t > 0) in its count,
+            // #(t < 0) below the parts that have arrived in its depth; the last one forms the result
+            unsigned long long* cl = reinterpret_cast<unsigned long long*>(&cell->depth);
+            unsigned long long* cg = reinterpret_cast<unsigned long long*>(&cell->count);
+            atomicAdd(cg, (unsigned long long)g);
+            __threadfence();
+            const unsigned long long was = atomicAdd(cl, (1ull << HD_PART_SHIFT) + (unsigned long long)l);
+            if ((int)(was >> HD_PART_SHIFT) != nparts - 1) return;
+            __threadfence();
+            l += (long long)(was & ((1ull << HD_PART_SHIFT) - 1));
+            g = (long long)atomicAdd(cg, 0ull);
+        }
+        const int64_t le = n - g, ge = n - l;
+        const int64_t c = le < ge ? le : ge;
+        *cell = ResDev{(double)c / (double)n, c};
     }
 }
 
-cudaError_t launch_hd_simt(const TaskDev* tasks, int ntasks, int max_ldx, const SlotDev* slots,
+cudaError_t launch_hd_simt(const TaskDev* tasks, int ntasks, int max_ldx, int64_t split_n, const SlotDev* slots,
                                const DsDev* ds, const float* U, const double* yz, const double* z64, ResDev* res,
                                int64_t* band_out, int* err, cudaStream_t st)
 {
     if (ntasks <= 0) return cudaSuccess;
-    const size_t smem = sizeof(float) * ((size_t)(HD_TJ + HD_PC) * max_ldx + HD_PC + HD_TJ);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_hd_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return e;
-        }
+    const size_t smem = sizeof(float) * ((size_t)HD_TJ * max_ldx + 2 * HD_K * HD_PC + 2 * HD_PC);
+    const cudaError_t e = cudaFuncSetAttribute(k_hd_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e;
     }
-    k_hd_simt<<<ntasks, HD_NT, smem, st>>>(tasks, slots, ds, U, yz, z64, res, band_out, err);
+    const dim3 grid((unsigned)ntasks, (unsigned)hd_parts(ntasks, split_n));
+    k_hd_simt<<<grid, HD_NT, smem, st>>>(tasks, slots, ds, U, yz, z64, res, band_out, err);
     return cudaGetLastError();
 }
 
