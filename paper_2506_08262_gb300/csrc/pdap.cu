@@ -28,7 +28,10 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "packed_fma.cuh"
+#include "pdap_common.cuh"
 #include "rrs_internal.h"
 
 namespace rrs {
@@ -36,21 +39,14 @@ namespace {
 
 constexpr int NT = 512;              // threads per CTA for G = 1, 2 (two CTAs per SM)
 constexpr int NT4 = 1024;            // threads per CTA for G = 4 (one CTA per SM)
-constexpr int NWARP = NT4 / 32;      // largest warp count of a CTA
 template <int G>
 __host__ __device__ constexpr int cta_threads()
 {
     return G == 4 ? NT4 : NT;
 }
-constexpr int NB = 2048;     // buckets per direction
-constexpr int CAP = 256;     // gathered keys per direction: the median run (and the D_AP MAD_+ run)
-constexpr int CAP1 = 512;    // second gather buffer: the D_AP MAD_+ run or the D_P MAD runs L, R
-constexpr int CAP1H = (NB - 256) / 2;   // D_P runs too large for it: pairs in the histogram area (after 256 counters)
 constexpr int MAXG = 4;
 // Stride of the resident keys of one direction in shared memory: n rounded up to 32 floats (128 bytes)
 __host__ __device__ constexpr int pdap_key_stride(int n) { return (n + 31) & ~31; }
-constexpr int FB_NB = NB;    // fallback histogram (reuses the bucket area)
-constexpr int FB_CAP = CAP + CAP1;  // fallback gather buffer: a direction's two gather areas
 
 // Per-direction constants and per-group scratch: after the projection pass,
 // group g (CTA threads / G) works on direction g alone and synchronises with
@@ -69,196 +65,6 @@ struct Ctl {
     int gn[MAXG];
     int gi[MAXG];                                         // smallest index of a tied run (fallback)
 };
-
-template <int GS>
-struct Grp {
-    int g, t;   // direction (group) index, thread index within the group
-    __device__ __forceinline__ void sync() const
-    {
-        if constexpr (GS == 32)
-            __syncwarp();   // one warp per direction: no named barrier needed
-        else
-            asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(GS) : "memory");
-    }
-};
-
-template <int NBK = NB>
-__device__ __forceinline__ int bucket(float y, float lo, float scale)
-{
-    // (y - lo) * scale, rounded once, truncated: monotone in y
-    const int b = __float2int_rz(__fmul_rn(__fsub_rn(y, lo), scale));
-    return b < 0 ? 0 : (b > NBK - 1 ? NBK - 1 : b);
-}
-
-// Bucket of the pass maps: y*sc + off rounded once, truncated (negatives saturate to 0),
-// clamped to the last bucket.  Monotone non-decreasing in y.
-template <int NBK = NB>
-__device__ __forceinline__ int bucket_fma(float y, float sc, float off)
-{
-    const unsigned b = __float2uint_rz(__fmaf_rn(y, sc, off));
-    return b < (unsigned)(NBK - 1) ? (int)b : NBK - 1;
-}
-
-// Bucket maps of k_pdap2: y*sc + off rounded once to an integer by the FMA itself.  o23 is off + 2^23,
-// so a result r in [2^23, 2^24) is an integer and its float bits are MAGIC + (r - 2^23).  bucket_raw
-// returns those bits as an int: non-decreasing in y for every result that is not a negative float, and
-// every negative float is a negative int.  bucket_m clamps them to [0, NBK): no float-to-integer
-// conversion, monotone non-decreasing in y.  A run of buckets [b1, b2] is the set of raw values in
-// [raw_lo(b1), raw_hi(b2)] (signed comparisons), the edge buckets taking every value clamped into them.
-constexpr int MAGIC = 0x4B000000;   // float bits of 2^23
-constexpr float TWO23 = 8388608.0f;
-__device__ __forceinline__ int bucket_raw(float y, float sc, float o23) { return __float_as_int(__fmaf_rn(y, sc, o23)); }
-template <int NBK = NB>
-__device__ __forceinline__ int bucket_m(float y, float sc, float o23)
-{
-    return min(max(bucket_raw(y, sc, o23), MAGIC), MAGIC + NBK - 1) - MAGIC;
-}
-template <int NBK = NB>
-__device__ __forceinline__ int raw_lo(int b)
-{
-    return b <= 0 ? INT_MIN : MAGIC + b;
-}
-template <int NBK = NB>
-__device__ __forceinline__ int raw_hi(int b)
-{
-    return b >= NBK - 1 ? INT_MAX : MAGIC + b;
-}
-
-__device__ __forceinline__ float warp_max(float v)
-{
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-    return v;
-}
-__device__ __forceinline__ float warp_min(float v)
-{
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) v = fminf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-    return v;
-}
-
-// Group sum of one int per thread (every thread gets the total).
-template <int GS, class CT>
-__device__ __forceinline__ int gsum(const Grp<GS>& q, int c, CT& C)
-{
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
-    if ((q.t & 31) == 0) C.red[q.g][q.t >> 5] = c;
-    q.sync();
-    int s = 0;
-#pragma unroll
-    for (int i = 0; i < GS / 32; ++i) s += C.red[q.g][i];
-    q.sync();
-    return s;
-}
-
-// Group min and max.
-template <int GS, class CT>
-__device__ void gminmax(const Grp<GS>& q, float lo, float hi, CT& C, float& olo, float& ohi)
-{
-    lo = warp_min(lo);
-    hi = warp_max(hi);
-    if ((q.t & 31) == 0) {
-        C.fred[q.g][q.t >> 5] = lo;
-        C.fred[q.g][NWARP + (q.t >> 5)] = hi;
-    }
-    q.sync();
-    olo = C.fred[q.g][0];
-    ohi = C.fred[q.g][NWARP];
-#pragma unroll
-    for (int i = 1; i < GS / 32; ++i) {
-        olo = fminf(olo, C.fred[q.g][i]);
-        ohi = fmaxf(ohi, C.fred[q.g][NWARP + i]);
-    }
-    q.sync();
-}
-
-// Group min and max of two pairs at once (one barrier round for both).
-template <int GS, class CT>
-__device__ __forceinline__ void gminmax2(const Grp<GS>& q, float& lo1, float& hi1, float& lo2, float& hi2, CT& C)
-{
-    constexpr int NW = GS / 32;   // at most 16: 4 NW values fit the 2 NWARP cells of fred
-    static_assert(4 * NW <= 2 * NWARP, "gminmax2 scratch");
-    lo1 = warp_min(lo1);
-    hi1 = warp_max(hi1);
-    lo2 = warp_min(lo2);
-    hi2 = warp_max(hi2);
-    const int w = q.t >> 5;
-    if ((q.t & 31) == 0) {
-        C.fred[q.g][w] = lo1;
-        C.fred[q.g][NW + w] = hi1;
-        C.fred[q.g][2 * NW + w] = lo2;
-        C.fred[q.g][3 * NW + w] = hi2;
-    }
-    q.sync();
-    lo1 = C.fred[q.g][0];
-    hi1 = C.fred[q.g][NW];
-    lo2 = C.fred[q.g][2 * NW];
-    hi2 = C.fred[q.g][3 * NW];
-#pragma unroll
-    for (int i = 1; i < NW; ++i) {
-        lo1 = fminf(lo1, C.fred[q.g][i]);
-        hi1 = fmaxf(hi1, C.fred[q.g][NW + i]);
-        lo2 = fminf(lo2, C.fred[q.g][2 * NW + i]);
-        hi2 = fmaxf(hi2, C.fred[q.g][3 * NW + i]);
-    }
-    q.sync();
-}
-
-// Exclusive scan of h[0..NB) by the group; the bucket holding rank ra and the
-// one holding rank rb (ra <= rb, both below the total), with the keys below each.
-template <int GS, class CT, int NBK = NB>
-__device__ void gfind(const Grp<GS>& q, const unsigned* h, int ra, int rb, CT& C, int& ba, int& ca, int& bb, int& cb)
-{
-    constexpr int PER = NBK / GS;   // 4 .. 32 consecutive buckets per thread, read as uint4
-    const int lane = q.t & 31, w = q.t >> 5;
-    int own = 0;
-    unsigned v[PER];
-    const uint4* h4 = reinterpret_cast<const uint4*>(h + q.t * PER);
-#pragma unroll
-    for (int k = 0; k < PER / 4; ++k) {
-        const uint4 a = h4[k];
-        v[4 * k] = a.x;
-        v[4 * k + 1] = a.y;
-        v[4 * k + 2] = a.z;
-        v[4 * k + 3] = a.w;
-    }
-#pragma unroll
-    for (int k = 0; k < PER; ++k) own += (int)v[k];
-    int incl = own;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) C.red[q.g][w] = incl;
-    q.sync();
-    int base = 0;
-#pragma unroll
-    for (int i = 0; i < GS / 32; ++i) base += i < w ? C.red[q.g][i] : 0;
-    int c = base + incl - own;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int hk = (int)v[k];
-        if (hk > 0) {
-            if (c <= ra && ra < c + hk) {
-                C.f_b1[q.g] = q.t * PER + k;
-                C.f_c1[q.g] = c;
-            }
-            if (c <= rb && rb < c + hk) {
-                C.f_b2[q.g] = q.t * PER + k;
-                C.f_c2[q.g] = c;
-            }
-        }
-        c += hk;
-    }
-    q.sync();
-    ba = C.f_b1[q.g];
-    ca = C.f_c1[q.g];
-    bb = C.f_b2[q.g];
-    cb = C.f_c2[q.g];
-    q.sync();
-}
 
 // One scan of h[0..NB) by the group locating the buckets of NR ranks rk[] (each below the total): for
 // each, the bucket, the keys below it and the keys in it.  With PREFIX, h becomes its inclusive prefix
@@ -322,212 +128,6 @@ __device__ __forceinline__ void gfindn(const Grp<GS>& q, unsigned* h, const int 
     q.sync();
 }
 
-// Values and point indices of the 0-based ranks s1 <= s2 among the pairs (buf, ib)[0..cnt), ordered by
-// value and then by point index, by the group.  The indices of one buffer are distinct, so every rank
-// names one pair and the choice among equal values never depends on the gather order.
-template <int GS, class CT>
-__device__ void gpick(const Grp<GS>& q, const float* buf, const int* ib, int cnt, int s1, int s2, CT& C, float& o1,
-                      float& o2, int& i1, int& i2)
-{
-    // tpk adjacent threads (one warp) rank one pair, each against every tpk-th pair, and add their counts:
-    // small sets are ranked in about cnt / tpk dependent steps.  Every thread of the group runs the same
-    // number of outer iterations, so the shuffles see whole warps.
-    const int tpk = cnt * 8 <= GS ? 8 : (cnt * 4 <= GS ? 4 : (cnt * 2 <= GS ? 2 : 1));
-    const int sub = q.t & (tpk - 1);
-    for (int t0 = 0; t0 < cnt; t0 += GS / tpk) {
-        const int t = t0 + q.t / tpk;
-        const bool live = t < cnt;
-        int r = 0;
-        float v = 0.f;
-        int iv = 0;
-        if (live) {
-            v = buf[t];
-            iv = ib[t];
-#pragma unroll 4
-            for (int s = sub; s < cnt; s += tpk) {
-                const float w2 = buf[s];
-                r += (w2 < v) | ((w2 == v) & (ib[s] < iv));
-            }
-        }
-        for (int o = 1; o < tpk; o <<= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, o);
-        if (live && sub == 0) {
-            if (r == s1) {
-                C.pv1[q.g] = v;
-                C.pi1[q.g] = iv;
-            }
-            if (r == s2) {
-                C.pv2[q.g] = v;
-                C.pi2[q.g] = iv;
-            }
-        }
-    }
-    q.sync();
-    o1 = C.pv1[q.g];
-    o2 = C.pv2[q.g];
-    i1 = C.pi1[q.g];
-    i2 = C.pi2[q.g];
-    q.sync();
-}
-
-// Ranks s1 <= s2 among the pairs (buf, ib)[0..cnt), every value in [lo, hi], ordered like gpick, for
-// sets too large for its all-pairs ranking: a 256-bucket histogram of the values (h2, 256 counters),
-// one warp's scan locates the buckets of the two ranks, their few pairs move to (tb, ti) and gpick ranks
-// them there.  Buckets are monotone in the value, so the rank of a pair is the count in lower buckets
-// plus its rank within its own bucket.
-constexpr int NB2 = 256;
-static_assert(NB2 + 2 * CAP1H == NB, "D_P runs in the histogram area: NB2 counters, then CAP1H values and CAP1H indices");
-template <int GS, class CT, int TCAP = CAP>
-__device__ void gpick_wide(const Grp<GS>& q, const float* buf, const int* ib, int cnt, int s1, int s2, float lo,
-                           float hi, unsigned* h2, float* tb, int* ti, CT& C, float& o1, float& o2, int& i1,
-                           int& i2)
-{
-    if (cnt <= 64 || !(lo < hi)) {
-        gpick(q, buf, ib, cnt, s1, s2, C, o1, o2, i1, i2);
-        return;
-    }
-    float scale = __fdiv_rn((float)NB2, __fsub_rn(hi, lo));
-    if (!(scale <= FLT_MAX)) scale = FLT_MAX;
-    for (int b = q.t; b < NB2; b += GS) h2[b] = 0u;
-    if (q.t == 0) C.gn[q.g] = 0;
-    q.sync();
-    auto bk = [&](float v) {
-        const int b = __float2int_rz(__fmul_rn(__fsub_rn(v, lo), scale));
-        return b < 0 ? 0 : (b > NB2 - 1 ? NB2 - 1 : b);
-    };
-    for (int t = q.t; t < cnt; t += GS) atomicAdd(&h2[bk(buf[t])], 1u);
-    q.sync();
-    if (q.t < 32) {
-        constexpr int PER2 = NB2 / 32;
-        const int lane = q.t;
-        unsigned v[PER2];
-        int own = 0;
-#pragma unroll
-        for (int k = 0; k < PER2; ++k) {
-            v[k] = h2[lane * PER2 + k];
-            own += (int)v[k];
-        }
-        int incl = own;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        int c = incl - own;
-#pragma unroll
-        for (int k = 0; k < PER2; ++k) {
-            const int hk = (int)v[k];
-            if (hk > 0) {
-                if (c <= s1 && s1 < c + hk) {
-                    C.f_b1[q.g] = lane * PER2 + k;
-                    C.f_c1[q.g] = c;
-                }
-                if (c <= s2 && s2 < c + hk) {
-                    C.f_b2[q.g] = lane * PER2 + k;
-                    C.f_c2[q.g] = c;
-                }
-            }
-            c += hk;
-        }
-    }
-    q.sync();
-    const int b1 = C.f_b1[q.g], c1 = C.f_c1[q.g], b2 = C.f_b2[q.g];
-    const int n2 = C.f_c2[q.g] + (int)h2[b2] - c1;
-    if (n2 > TCAP) {   // the rank buckets hold more pairs than (tb, ti): rank the whole set
-        gpick(q, buf, ib, cnt, s1, s2, C, o1, o2, i1, i2);
-        return;
-    }
-    for (int t = q.t; t < cnt; t += GS) {
-        const float v = buf[t];
-        const int b = bk(v);
-        if (b >= b1 && b <= b2) {
-            const int pos = atomicAdd(&C.gn[q.g], 1);
-            if (pos < TCAP) {
-                tb[pos] = v;
-                ti[pos] = ib[t];
-            }
-        }
-    }
-    q.sync();
-    gpick(q, tb, ti, n2, s1 - c1, s2 - c1, C, o1, o2, i1, i2);
-}
-
-// Generic exact selection of ranks q1 <= q2 over one direction's values f(0..L-1),
-// all in [lo, hi], by iterated bucketing (the fallback path); hist, buf and ibuf are the
-// direction's own areas.  Returns the values and the point indices of the two ranks.
-template <int GS, class CT, class F, int FBN = FB_NB, int FBC = FB_CAP>
-__device__ void gselect(const Grp<GS>& q, F f, int L, int q1, int q2, float lo, float hi, unsigned* hist, float* buf,
-                        int* ibuf, CT& C, float& v1, float& v2, int& i1, int& i2, int* err)
-{
-    int below = 0;
-    for (int iter = 0; iter < 24; ++iter) {
-        if (!(lo < hi)) {
-            // every remaining candidate equals lo: both ranks hold that value, taken at the
-            // smallest point index that holds it
-            if (q.t == 0) C.gi[q.g] = 0x7FFFFFFF;
-            q.sync();
-            for (int i = q.t; i < L; i += GS) {
-                if (f(i) == lo) {
-                    atomicMin(&C.gi[q.g], i);
-                    break;
-                }
-            }
-            q.sync();
-            v1 = v2 = lo;
-            i1 = i2 = C.gi[q.g];
-            q.sync();
-            return;
-        }
-        float scale = __fdiv_rn((float)FBN, __fsub_rn(hi, lo));
-        if (!(scale <= FLT_MAX)) scale = FLT_MAX;
-        for (int b = q.t; b < FBN / 4; b += GS) reinterpret_cast<uint4*>(hist)[b] = make_uint4(0u, 0u, 0u, 0u);
-        q.sync();
-        for (int i = q.t; i < L; i += GS) {
-            const float a = f(i);
-            if (a >= lo && a <= hi) atomicAdd(&hist[bucket<FBN>(a, lo, scale)], 1u);
-        }
-        q.sync();
-        int b1, c1, b2, c2;
-        gfind<GS, CT, FBN>(q, hist, q1 - below, q2 - below, C, b1, c1, b2, c2);
-        const int cnt = c2 + (int)hist[b2] - c1;
-        if (q.t == 0) C.gn[q.g] = 0;
-        q.sync();
-        if (cnt <= FBC) {
-            for (int i = q.t; i < L; i += GS) {
-                const float a = f(i);
-                if (a >= lo && a <= hi) {
-                    const int b = bucket<FBN>(a, lo, scale);
-                    if (b >= b1 && b <= b2) {
-                        const int pos = atomicAdd(&C.gn[q.g], 1);
-                        if (pos < FBC) {
-                            buf[pos] = a;
-                            ibuf[pos] = i;
-                        }
-                    }
-                }
-            }
-            q.sync();
-            gpick(q, buf, ibuf, cnt, q1 - below - c1, q2 - below - c1, C, v1, v2, i1, i2);
-            return;
-        }
-        float nlo = FLT_MAX, nhi = -FLT_MAX;
-        for (int i = q.t; i < L; i += GS) {
-            const float a = f(i);
-            if (a >= lo && a <= hi) {
-                const int b = bucket<FBN>(a, lo, scale);
-                if (b >= b1 && b <= b2) {
-                    nlo = fminf(nlo, a);
-                    nhi = fmaxf(nhi, a);
-                }
-            }
-        }
-        gminmax(q, nlo, nhi, C, lo, hi);
-        below += c1;
-    }
-    if (q.t == 0) atomicOr(err, ERR_SELECT_ITER);
-    v1 = v2 = __int_as_float(0x7FC00000);
-    i1 = i2 = -1;
-}
-
 // 1 / (1 + num / spread) = spread / (spread + num) for num, spread >= 0 (FP64 inputs, exact differences
 // of FP32 order statistics).  GB300 issues FP64 at a fraction of the FP32 rate, so the one division is
 // done in FP32 (relative error a few 2^-24) whenever both operands and the quotient are safely normal
@@ -555,91 +155,52 @@ __device__ __forceinline__ float key_halves(const float* u, const float* x)
     return __fadd_rn(p0, p1);
 }
 
-// Row i of X as D4 floats (D4 <= ldx, the padding zero): from the dataset's tiled copy Xt when it keeps
-// one, else from the padded rows; the same values either way.  The projection pass streams X once per CTA
-// and is bound by the cache lines its loads touch: a warp reading chunk c of 32 consecutive rows reads 512
-// contiguous bytes of Xt, where in the padded rows the same 32 chunks lie on every line of the 32 rows.
-template <int D4>
-__device__ __forceinline__ void load_row(const DsDev& D, int i, int ldx, float (&xv)[D4])
-{
-    const float4* xr = D.Xt ? reinterpret_cast<const float4*>(D.Xt) + ((int64_t)(i >> 5) * (ldx >> 2)) * 32 + (i & 31)
-                            : reinterpret_cast<const float4*>(D.X32 + (int64_t)i * ldx);
-    const int cs = D.Xt ? 32 : 1;   // float4 stride between the chunks of one row
-#pragma unroll
-    for (int c = 0; c < D4 / 4; ++c) {
-        const float4 t4 = xr[c * cs];
-        xv[4 * c] = t4.x;
-        xv[4 * c + 1] = t4.y;
-        xv[4 * c + 2] = t4.z;
-        xv[4 * c + 3] = t4.w;
-    }
-}
-
 // Pass A of k_pdap2 for d <= 16 (D4 = d rounded up to 4, the directions uu in registers): the keys of G
-// directions for the points i = tid + k NTK, stored (unless STREAM) and counted in the directions' histograms.
-// xp points at row tid; CS is the float4 distance between the 16-byte chunks of one row (32 in the tiled
-// copy Xt, 1 in the padded rows).  In both layouts rows i and i + NTK lie rstep = NTK ldx / 4 float4 apart
-// (NTK is a multiple of 32, so i mod 32 stays put within a tile), so a thread walks its rows by a pointer
-// increment and every chunk load takes a constant offset.  Two rows per iteration keep six loads in flight.
-template <int G, int D4, bool STREAM, int CS, int NTK>
-__device__ __forceinline__ void pass_a_rows(const float4* __restrict__ xp, size_t rstep, int tid, int n, int kst,
-                                            const float (&uu)[G][D4], const float (&sc)[G], const float (&of)[G],
-                                            float* keys, unsigned* hist)
+// directions for the points t0, t0 + 1, then step further on, stored (unless STREAM) and counted in the
+// directions' histograms.  Two points per thread: from the dataset's columns Xt (dim l of point i at
+// l * colst + i) their coordinates come as one 8-byte load per dim, side by side over the lanes; without columns
+// from the padded rows.
+template <int G, int D4, bool STREAM>
+__device__ __forceinline__ void pass_a_pairs(const DsDev& D, int t0, int step, int n, int kst, const float (&uu)[G][D4],
+                                             const float (&sc)[G], const float (&of)[G], float* keys, unsigned* hist)
 {
-    float* kq = keys + tid;   // key of direction g for the thread's current row: kq[g * kst]
-    int i = tid;
-    for (; i + NTK < n; i += 2 * NTK, xp += 2 * rstep, kq += 2 * NTK) {
-        const float4* xq = xp + rstep;
+    const size_t colst = (size_t)((n + 31) & ~31);
+    for (unsigned i = t0; i < (unsigned)n; i += step) {
+        const bool two = i + 1 < (unsigned)n;
         float xa[D4], xb[D4];
+        if (D.Xt) {
 #pragma unroll
-        for (int c = 0; c < D4 / 4; ++c) {
-            const float4 a = xp[c * CS], b = xq[c * CS];
-            xa[4 * c] = a.x;
-            xa[4 * c + 1] = a.y;
-            xa[4 * c + 2] = a.z;
-            xa[4 * c + 3] = a.w;
-            xb[4 * c] = b.x;
-            xb[4 * c + 1] = b.y;
-            xb[4 * c + 2] = b.z;
-            xb[4 * c + 3] = b.w;
+            for (int l = 0; l < D4; ++l) {
+                float2 v = make_float2(0.f, 0.f);
+                if (l < D.d) v = *reinterpret_cast<const float2*>(D.Xt + l * colst + i);
+                xa[l] = v.x;
+                xb[l] = v.y;
+            }
+        } else {
+            const float4* ra = reinterpret_cast<const float4*>(D.X32 + (int64_t)i * D.ldx);
+            const float4* rb = reinterpret_cast<const float4*>(D.X32 + (int64_t)(two ? i + 1 : i) * D.ldx);
+#pragma unroll
+            for (int c = 0; c < D4 / 4; ++c) {
+                const float4 a = ra[c], b = rb[c];
+                xa[4 * c] = a.x;
+                xa[4 * c + 1] = a.y;
+                xa[4 * c + 2] = a.z;
+                xa[4 * c + 3] = a.w;
+                xb[4 * c] = b.x;
+                xb[4 * c + 1] = b.y;
+                xb[4 * c + 2] = b.z;
+                xb[4 * c + 3] = b.w;
+            }
         }
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             const float ka = key_halves<D4>(uu[g], xa), kb = key_halves<D4>(uu[g], xb);
-            if (!STREAM) {
-                kq[g * kst] = ka;
-                kq[g * kst + NTK] = kb;
-            }
+            if (!STREAM) *reinterpret_cast<float2*>(keys + (size_t)g * kst + i) = make_float2(ka, kb);   // kst is even
             atomicAdd(&hist[g * NB + bucket_m(ka, sc[g], of[g])], 1u);
-            atomicAdd(&hist[g * NB + bucket_m(kb, sc[g], of[g])], 1u);
-        }
-    }
-    if (i < n) {
-        float xa[D4];
-#pragma unroll
-        for (int c = 0; c < D4 / 4; ++c) {
-            const float4 a = xp[c * CS];
-            xa[4 * c] = a.x;
-            xa[4 * c + 1] = a.y;
-            xa[4 * c + 2] = a.z;
-            xa[4 * c + 3] = a.w;
-        }
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const float ka = key_halves<D4>(uu[g], xa);
-            if (!STREAM) kq[g * kst] = ka;
-            atomicAdd(&hist[g * NB + bucket_m(ka, sc[g], of[g])], 1u);
+            if (two) atomicAdd(&hist[g * NB + bucket_m(kb, sc[g], of[g])], 1u);
         }
     }
 }
-
-// One direction's keys held in an array: shared memory (resident keys) or device memory (keys formed
-// by launch_pdap_keys when they do not fit shared memory).
-struct KeysArray {
-    const float* y;
-    __device__ __forceinline__ float get(int i) const { return y[i]; }
-    __device__ __forceinline__ float4 get4(int i) const { return *reinterpret_cast<const float4*>(y + i); }
-};
 
 // One direction's keys recomputed from the FP32 rows of X with the projection pass's arithmetic
 // (two half chains for d <= 16, one sequential FMA chain otherwise), so every pass sees the values
@@ -724,38 +285,6 @@ __device__ __forceinline__ void mad_runs(const Grp<GS>& q, unsigned* H, CT& C, i
     }
 }
 
-// D_P's MAD from the gathered runs L, R (keys B1[0..cnt1), point indices I1) once the median m is known:
-// the deviations replace the keys in place and the ranks s1 <= s2 among them are picked (gpick_wide, with
-// h2 and the TCAP pairs tb / ti as scratch).  Every key between the runs lies in (max L, min R) and every
-// key outside them below min L or above max R, so the picks are the MAD ranks of all keys when the
-// deviations those bounds allow do not cross them; returns whether they do not (else nothing is picked
-// for sure and the caller takes the |y - med| histogram pass).
-template <int GS, int TCAP, class CT>
-__device__ bool mad_from_runs(const Grp<GS>& q, float* B1, int* I1, int cnt1, int s1, int s2, float m, unsigned* h2,
-                              float* tb, int* ti, CT& C, float& p1, float& p2, int& ip1, int& ip2)
-{
-    float lmin = FLT_MAX, lmax = -FLT_MAX, rmin = FLT_MAX, rmax = -FLT_MAX;
-    for (int t = q.t; t < cnt1; t += GS) {
-        const float v = B1[t];
-        if (v < m) {   // L keys lie below m1 <= m, R keys above m2 >= m
-            lmin = fminf(lmin, v);
-            lmax = fmaxf(lmax, v);
-        } else {
-            rmin = fminf(rmin, v);
-            rmax = fmaxf(rmax, v);
-        }
-        B1[t] = fabsf(__fsub_rn(v, m));
-    }
-    gminmax2(q, lmin, lmax, rmin, rmax, C);
-    const float la = lmin, lb = lmax, ra = rmin, rb = rmax;
-    if (!(lb > -FLT_MAX && ra < FLT_MAX && s1 >= 0 && s2 < cnt1)) return false;
-    const float inner = fmaxf(__fsub_rn(m, lb), __fsub_rn(ra, m));
-    const float outer = fminf(__fsub_rn(m, la), __fsub_rn(rb, m));
-    gpick_wide<GS, CT, TCAP>(q, B1, I1, cnt1, s1, s2, fminf(__fsub_rn(m, lb), __fsub_rn(ra, m)),
-                             fmaxf(__fsub_rn(m, la), __fsub_rn(rb, m)), h2, tb, ti, C, p1, p2, ip1, ip2);
-    return inner <= p1 && outer >= p2;
-}
-
 // FP64 projection u'x_i of point i: one sequential FMA chain over the dims, from the FP64 rows when
 // the data came in FP64 (the direction generator forms the query's y_z = u'z the same way, so a query
 // equal to a data point projects to the same value).  Every product of an FP32 direction component and
@@ -771,19 +300,6 @@ __device__ __forceinline__ double proj64(const DsDev& D, const float* u, int i)
         for (int l = 0; l < D.d; ++l) acc = __fma_rn((double)u[l], (double)xr[l], acc);
     }
     return acc;
-}
-
-// The points a selection kernel picked for one direction are written into the direction's result cell in
-// place of its depth, which k_pdap_finish then forms from them: the points of the median ranks (im1, im2)
-// and of the MAD or MAD_+ ranks (ip1, ip2); -1 where a selection failed (its error flag is set), and
-// ip1 = ip2 = NOPOS for D_AP when no key lies above the median (MAD_+ = 0).  Two 8-byte stores: a result
-// cell is 8-byte aligned.
-constexpr int NOPOS = -2;
-__device__ __forceinline__ void put_picks(ResDev* cell, int im1, int im2, int ip1, int ip2)
-{
-    int2* c = reinterpret_cast<int2*>(cell);
-    c[0] = make_int2(im1, im2);
-    c[1] = make_int2(ip1, ip2);
 }
 
 // FP64 finish of a selection launch: the depth of every direction from its picks (put_picks).  Four
@@ -824,7 +340,7 @@ __global__ void __launch_bounds__(256) k_pdap_finish(const TaskDev* __restrict__
         ap = S.kind == 2;
         yzv = yz[S.roff + T.j0 + g];
         const int sel = k == 0 ? a.x : (k == 1 ? a.y : (k == 2 ? b.x : b.y));
-        if (sel >= 0) y = proj64(D, U + S.uoff + (int64_t)(T.j0 + g) * D.ldx, sel);
+        if (sel >= 0 && sel < D.n) y = proj64(D, U + S.uoff + (int64_t)(T.j0 + g) * D.ldx, sel);
     }
     // every lane of the warp takes part in the shuffles; the four lanes of a direction are adjacent
     const int lane = threadIdx.x & 31, l0 = lane & ~3;
@@ -1250,16 +766,15 @@ __global__ void __launch_bounds__(cta_threads<G>(), (G >= 4 ? 1 : 2)) k_pdap2(co
                 ua[l] = uS[(2 * pair) * ldx + l];
                 ub[l] = uS[(2 * pair + 1) * ldx + l];
             }
-            const float sca = sc[2 * pair], ofa = of[2 * pair], scb = sc[2 * pair + 1], ofb = of[2 * pair + 1];
-            for (int i = tid >> 1; i < n; i += NTK / 2) {
-                float xv[D4];
-                load_row<D4>(D, i, ldx, xv);
-                const float ka = key_halves<D4>(ua, xv), kb = key_halves<D4>(ub, xv);
-                if (!STREAM) keys[(size_t)(2 * pair) * kst + i] = ka;
-                atomicAdd(&hist[(2 * pair) * NB + bucket_m(ka, sca, ofa)], 1u);
-                if (!STREAM) keys[(size_t)(2 * pair + 1) * kst + i] = kb;
-                atomicAdd(&hist[(2 * pair + 1) * NB + bucket_m(kb, scb, ofb)], 1u);
+            float u2[2][D4];
+#pragma unroll
+            for (int l = 0; l < D4; ++l) {
+                u2[0][l] = ua[l];
+                u2[1][l] = ub[l];
             }
+            const float s2[2] = {sc[2 * pair], sc[2 * pair + 1]}, o2[2] = {of[2 * pair], of[2 * pair + 1]};
+            pass_a_pairs<2, D4, STREAM>(D, 2 * (tid >> 1), NTK, n, kst, u2, s2, o2, keys + (size_t)(2 * pair) * kst,
+                                        hist + 2 * pair * NB);
         } else if (DP4 > 0) {
             constexpr int D4 = DP4 > 0 ? DP4 : 4;
             float uu[G][D4];
@@ -1273,15 +788,7 @@ __global__ void __launch_bounds__(cta_threads<G>(), (G >= 4 ? 1 : 2)) k_pdap2(co
                     uu[g][4 * c + 2] = u4.z;
                     uu[g][4 * c + 3] = u4.w;
                 }
-            const int c4 = ldx >> 2;
-            const size_t rstep = (size_t)NTK * c4;
-            if (D.Xt)
-                pass_a_rows<G, D4, STREAM, 32, NTK>(reinterpret_cast<const float4*>(D.Xt) +
-                                                        ((size_t)(tid >> 5) * c4 * 32 + (tid & 31)),
-                                                    rstep, tid, n, kst, uu, sc, of, keys, hist);
-            else
-                pass_a_rows<G, D4, STREAM, 1, NTK>(reinterpret_cast<const float4*>(D.X32) + (size_t)tid * c4, rstep,
-                                                   tid, n, kst, uu, sc, of, keys, hist);
+            pass_a_pairs<G, D4, STREAM>(D, 2 * tid, 2 * NTK, n, kst, uu, sc, of, keys, hist);
         } else {
             for (int i = tid; i < n; i += NTK) {
                 const float4* xr = reinterpret_cast<const float4*>(D.X32 + (int64_t)i * ldx);
@@ -1306,572 +813,6 @@ __global__ void __launch_bounds__(cta_threads<G>(), (G >= 4 ? 1 : 2)) k_pdap2(co
     __syncthreads();
 
     select_dirs<G, DP4, STREAM>(C, keys, uS, hist, buf, ibuf, n, npad, kst, ap, D, GA, S.roff + T.j0, res, err, kin);
-}
-
-// ---------------------------------------------------------------------------------------------
-// Warp-per-direction selection, keys recomputed from X at every pass (d <= 16, n <= PDAPW_MAX_N)
-// ---------------------------------------------------------------------------------------------
-// One CTA of WPC warps takes up to WPC directions of one query; warp w owns direction w.  No key is
-// stored: pass A (the whole CTA, one X row per thread, every direction) forms each key and counts it
-// in its direction's histogram (16-bit counters, two per word); each warp then finds its runs (the
-// median run and, in the same pass, the D_P MAD runs or the D_AP MAD_+ run, as in select_dir); the
-// gather pass (the whole CTA again) re-forms every key with the same arithmetic and moves the keys of
-// the runs, with their point indices, into the warps' buffers; each warp ranks its buffers and forms
-// the depth from FP64 projections of the selected points.  X is read twice per WPC directions, the
-// selection work of a direction stays inside its warp (no block barrier), and the key arithmetic is
-// that of the other selection kernels, so every kernel selects the same points.
-constexpr int WPC = PDAPW_DIRS;    // directions (warps) per CTA
-constexpr int WNB = 2048;          // buckets per direction (16-bit counters, WNB / 2 words)
-constexpr int WCAP0 = 128;         // median-run buffer
-constexpr int WCAP1 = 448;         // MAD_+ run or MAD L, R runs buffer
-constexpr int WFBN = 1024;         // fallback histogram: 32-bit counters in the same WNB / 2 words
-constexpr int WNT = WPC * 32;
-
-struct CtlW {
-    float lo_b[WPC], sc_y[WPC], off_y[WPC], scale[WPC];
-    int red[WPC][2];
-    float fred[WPC][2 * NWARP];
-    int fill[WPC][2];
-    int f_b1[WPC], f_c1[WPC], f_b2[WPC], f_c2[WPC];
-    float pv1[WPC], pv2[WPC];
-    int pi1[WPC], pi2[WPC];
-    int gn[WPC], gi[WPC];
-    // gather-pass tests of every direction: bucket map (sc, off), median run [bl0, bl0 + bw0], second set
-    // |2b - c2| in [dl2, dl2 + dw2]
-    float4 pa[WPC];
-    int4 pb[WPC];
-    // deviation passes of D_P directions: (med, bucket scale, run start or OFF (0 before the run is known), run width)
-    float4 dv[WPC];
-    int ndev;
-};
-
-// Key of a point for exactly D dims: the two half chains of key_halves<DP4> without their zero-padded
-// terms (a zero product leaves a chain unchanged), so the values are those of the other kernels.
-template <int D>
-__device__ __forceinline__ float key_w(const float* u, const float* x)
-{
-    constexpr int DP4 = (D + 3) & ~3, H2 = DP4 / 2, E0 = D < H2 ? D : H2;
-    float p0 = 0.f, p1 = 0.f;
-#pragma unroll
-    for (int l = 0; l < E0; ++l) p0 = fmaf(u[l], x[l], p0);
-#pragma unroll
-    for (int l = H2; l < D; ++l) p1 = fmaf(u[l], x[l], p1);
-    return __fadd_rn(p0, p1);
-}
-
-// The warp's histogram words are stored transposed: word v (of 1,024) at (v mod 32) * 32 + v / 32, so
-// when lane l walks words 32 l .. 32 l + 31 (its range of buckets) the 32 lanes read 32 banks.
-__device__ __forceinline__ int hidx(int v) { return ((v & 31) << 5) | (v >> 5); }
-__device__ __forceinline__ void h16_add(unsigned* h, int b) { atomicAdd(&h[hidx(b >> 1)], 1u << ((b & 1) << 4)); }
-__device__ __forceinline__ int h16_get(const unsigned* h, int b)
-{
-    return (int)((h[hidx(b >> 1)] >> ((b & 1) << 4)) & 0xFFFFu);
-}
-
-// Buckets holding ranks ra <= rb (both below the total) of a transposed warp histogram, and the counts
-// below each, by one warp.  P16: 2,048 buckets of 16-bit counters (two per word), else 1,024 buckets of
-// 32-bit counters.  Lane l owns words 32 l .. 32 l + 31.
-template <bool P16>
-__device__ void wfind(const unsigned* h, int ra, int rb, int& ba, int& ca, int& bb, int& cb)
-{
-    const int lane = threadIdx.x & 31;
-    int own = 0;
-#pragma unroll 8
-    for (int j = 0; j < 32; ++j) {
-        const unsigned wd = h[(j << 5) | lane];
-        own += P16 ? (int)((wd & 0xFFFFu) + (wd >> 16)) : (int)wd;
-    }
-    int incl = own;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    int c = incl - own, fa = -1, fca = 0, fb = -1, fcb = 0;
-    const bool mine = (c <= rb && ra < c + own);   // only lanes whose range meets [ra, rb] walk it
-    if (mine) {
-#pragma unroll 1
-        for (int j = 0; j < 32; ++j) {
-            const unsigned wd = h[(j << 5) | lane];
-#pragma unroll
-            for (int hh = 0; hh < (P16 ? 2 : 1); ++hh) {
-                const int hk = P16 ? (int)((wd >> (16 * hh)) & 0xFFFFu) : (int)wd;
-                const int b = P16 ? lane * 64 + 2 * j + hh : lane * 32 + j;
-                if (hk > 0) {
-                    if (c <= ra && ra < c + hk) {
-                        fa = b;
-                        fca = c;
-                    }
-                    if (c <= rb && rb < c + hk) {
-                        fb = b;
-                        fcb = c;
-                    }
-                }
-                c += hk;
-            }
-        }
-    }
-    const int la = __ffs(__ballot_sync(0xFFFFFFFFu, fa >= 0)) - 1, lb = __ffs(__ballot_sync(0xFFFFFFFFu, fb >= 0)) - 1;
-    ba = __shfl_sync(0xFFFFFFFFu, fa, la);
-    ca = __shfl_sync(0xFFFFFFFFu, fca, la);
-    bb = __shfl_sync(0xFFFFFFFFu, fb, lb);
-    cb = __shfl_sync(0xFFFFFFFFu, fcb, lb);
-}
-
-// Inclusive prefix counts of a transposed 16-bit warp histogram in place (every count, and n, below 2^16).
-__device__ void wprefix(unsigned* h)
-{
-    const int lane = threadIdx.x & 31;
-    int own = 0;
-#pragma unroll 8
-    for (int j = 0; j < 32; ++j) {
-        const unsigned wd = h[(j << 5) | lane];
-        own += (int)((wd & 0xFFFFu) + (wd >> 16));
-    }
-    int incl = own;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    unsigned run = (unsigned)(incl - own);
-#pragma unroll 8
-    for (int j = 0; j < 32; ++j) {
-        const unsigned wd = h[(j << 5) | lane];
-        const unsigned lo = run + (wd & 0xFFFFu), hi = lo + (wd >> 16);
-        run = hi;
-        h[(j << 5) | lane] = lo | (hi << 16);
-    }
-    __syncwarp();
-}
-
-// Prefix count through bucket b (0 for b < 0) of a histogram turned into prefix counts by wprefix.
-__device__ __forceinline__ int wP(const unsigned* h, int b) { return b < 0 ? 0 : h16_get(h, b); }
-
-// One direction's keys re-formed from X (the gather-pass arithmetic), for the warp's fallback passes.
-template <int D>
-struct KeysW {
-    const float* X;
-    const float* u;
-    int ldx;
-    __device__ __forceinline__ float get(int i) const
-    {
-        constexpr int DP4 = (D + 3) & ~3;
-        const float4* xr = reinterpret_cast<const float4*>(X + (int64_t)i * ldx);
-        float xv[DP4], uv[DP4];
-#pragma unroll
-        for (int c = 0; c < DP4 / 4; ++c) {
-            const float4 t4 = xr[c];
-            const float4 u4 = *reinterpret_cast<const float4*>(u + 4 * c);
-            xv[4 * c] = t4.x;
-            xv[4 * c + 1] = t4.y;
-            xv[4 * c + 2] = t4.z;
-            xv[4 * c + 3] = t4.w;
-            uv[4 * c] = u4.x;
-            uv[4 * c + 1] = u4.y;
-            uv[4 * c + 2] = u4.z;
-            uv[4 * c + 3] = u4.w;
-        }
-        return key_w<D>(uv, xv);
-    }
-};
-
-// Ranks s1 <= s2 of the pairs (buf, ib)[0..cnt): all-pairs ranking for small sets, else the value range
-// and gpick_wide (h2: NB2 words, tb / ti: TCAP pairs of scratch).
-template <int GS, int TCAP, class CT>
-__device__ void gpick_auto(const Grp<GS>& q, const float* buf, const int* ib, int cnt, int s1, int s2, unsigned* h2,
-                           float* tb, int* ti, CT& C, float& o1, float& o2, int& i1, int& i2)
-{
-    if (cnt <= 64) {
-        gpick(q, buf, ib, cnt, s1, s2, C, o1, o2, i1, i2);
-        return;
-    }
-    float lo = FLT_MAX, hi = -FLT_MAX;
-    for (int t = q.t; t < cnt; t += GS) {
-        lo = fminf(lo, buf[t]);
-        hi = fmaxf(hi, buf[t]);
-    }
-    gminmax(q, lo, hi, C, lo, hi);
-    gpick_wide<GS, CT, TCAP>(q, buf, ib, cnt, s1, s2, lo, hi, h2, tb, ti, C, o1, o2, i1, i2);
-}
-
-// The warp's last part: the iterated-bucket fallbacks over re-formed keys where a run overflowed its
-// buffer (fb = 1: every statistic; fb = 2: the spread only), then the picks (as in select_dir).
-template <int D>
-__device__ void close_warp(const Grp<32>& q, const KeysW<D>& y, CtlW& C, unsigned* H, float* B0, int* I0, int n,
-                           bool ap, int fb, float m1, float m2, int im1, int im2, float p1, float p2, int ip1, int ip2,
-                           int npos, ResDev* __restrict__ out, int* err)
-{
-    const int k1 = (n - 1) / 2, k2 = n / 2;
-    if (fb) {
-        float kl = FLT_MAX, kh = -FLT_MAX;
-        for (int i = q.t; i < n; i += 32) {
-            const float v = y.get(i);
-            kl = fminf(kl, v);
-            kh = fmaxf(kh, v);
-        }
-        gminmax(q, kl, kh, C, kl, kh);
-        auto f = [&](int i) { return y.get(i); };
-        if (fb == 1)
-            gselect<32, CtlW, decltype(f), WFBN, WCAP0 + WCAP1>(q, f, n, k1, k2, kl, kh, H, B0, I0, C, m1, m2, im1,
-                                                                im2, err);
-        if (ap) {
-            int c = 0;
-            for (int i = q.t; i < n; i += 32) c += (y.get(i) <= m1);
-            const int nle = gsum(q, c, C);
-            npos = n - nle;
-            ip1 = ip2 = -1;
-            if (npos > 0)
-                gselect<32, CtlW, decltype(f), WFBN, WCAP0 + WCAP1>(q, f, n, nle + (npos - 1) / 2, nle + npos / 2, kl,
-                                                                    kh, H, B0, I0, C, p1, p2, ip1, ip2, err);
-        } else {
-            const float m = __fmul_rn(__fadd_rn(m1, m2), 0.5f);
-            const float dmax = fmaxf(fabsf(__fsub_rn(kl, m)), fabsf(__fsub_rn(kh, m)));
-            auto fd = [&](int i) { return fabsf(__fsub_rn(y.get(i), m)); };
-            gselect<32, CtlW, decltype(fd), WFBN, WCAP0 + WCAP1>(q, fd, n, k1, k2, 0.0f, dmax, H, B0, I0, C, p1, p2,
-                                                                 ip1, ip2, err);
-        }
-    }
-    if (q.t == 0) put_picks(out, im1, im2, ap && npos == 0 ? NOPOS : ip1, ap && npos == 0 ? NOPOS : ip2);
-}
-
-template <int D>
-__global__ void __launch_bounds__(WNT, 2) k_pdapw(const TaskDev* __restrict__ tasks, const SlotDev* __restrict__ slots,
-                                                   const DsDev* __restrict__ dsets, const float* __restrict__ U,
-                                                   ResDev* __restrict__ res, int* err)
-{
-    constexpr int DP4 = (D + 3) & ~3;
-    constexpr int OFF = 1 << 30;
-    extern __shared__ __align__(16) float smw[];
-    __shared__ CtlW C;
-    const TaskDev T = tasks[blockIdx.x];
-    const SlotDev& S = slots[T.slot];
-    const DsDev Dd = dsets[S.ds];
-    const int n = (int)Dd.n, ldx = Dd.ldx, d = Dd.d;
-    const bool ap = (S.kind == 2);
-    const int GA = T.nj;   // live directions; warps GA..WPC-1 are inert
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    float* uS = smw;                                                       // WPC x DP4
-    unsigned* hist = reinterpret_cast<unsigned*>(uS + WPC * DP4);          // WPC x WNB / 2 words
-    float* bufB = reinterpret_cast<float*>(hist + WPC * (WNB / 2));        // WPC x (WCAP0 + WCAP1)
-    int* bufI = reinterpret_cast<int*>(bufB + WPC * (WCAP0 + WCAP1));      // WPC x (WCAP0 + WCAP1)
-    for (int e = tid; e < WPC * DP4; e += WNT) {
-        const int g = e / DP4, l = e - g * DP4;
-        uS[e] = (g < GA && l < d) ? U[S.uoff + (int64_t)(T.j0 + g) * ldx + l] : 0.0f;
-    }
-    for (int e = tid; e < WPC * WNB / 8; e += WNT) reinterpret_cast<uint4*>(hist)[e] = make_uint4(0u, 0u, 0u, 0u);
-    if (tid == 0) C.ndev = 0;
-    __syncthreads();
-    // bucket range of direction w (as k_pdap2): the centre's projection +- 5 sigma_u, or +- the radius
-    if (w < GA) {
-        const float* u = uS + w * DP4;
-        float yc = 0.0f, qf = 0.0f;
-        for (int r = lane; r < d; r += 32) yc = fmaf(u[r], Dd.center[r], yc);
-        if (Dd.cov) {
-            for (int e = lane; e < d * d; e += 32) {
-                const int r = e / d, c2 = e - r * d;
-                qf = fmaf(Dd.cov[e], __fmul_rn(u[r], u[c2]), qf);
-            }
-        }
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-            yc += __shfl_xor_sync(0xFFFFFFFFu, yc, o);
-            qf += __shfl_xor_sync(0xFFFFFFFFu, qf, o);
-        }
-        if (lane == 0) {
-            float half = Dd.rc * 1.0001f;
-            if (Dd.cov) {
-                const float sg = sqrtf(fmaxf(qf, 0.0f));
-                if (sg > 0.0f && 5.0f * sg < half) half = 5.0f * sg;
-                C.scale[w] = sg;
-            } else {
-                C.scale[w] = half;
-            }
-            if (!(half > 0.0f)) half = fmaxf(fabsf(yc), 1.0f);
-            C.lo_b[w] = yc - half;
-            C.sc_y[w] = __fdiv_rn((float)WNB, __fadd_rn(half, half));
-            C.off_y[w] = __fmul_rn(-C.lo_b[w], C.sc_y[w]);
-        }
-    }
-    __syncthreads();
-
-    // two rows per thread and iteration: the row loads of both are in flight together, and each direction's
-    // vector is read from shared memory once for the two keys
-    auto rows = [&](int i, float (&xa)[DP4], float (&xb)[DP4], bool two, int i2) {
-        const float4* ra = reinterpret_cast<const float4*>(Dd.X32 + (int64_t)i * ldx);
-        const float4* rb = reinterpret_cast<const float4*>(Dd.X32 + (int64_t)(two ? i2 : i) * ldx);
-#pragma unroll
-        for (int c = 0; c < DP4 / 4; ++c) {
-            const float4 a = ra[c], b = rb[c];
-            xa[4 * c] = a.x;
-            xa[4 * c + 1] = a.y;
-            xa[4 * c + 2] = a.z;
-            xa[4 * c + 3] = a.w;
-            xb[4 * c] = b.x;
-            xb[4 * c + 1] = b.y;
-            xb[4 * c + 2] = b.z;
-            xb[4 * c + 3] = b.w;
-        }
-    };
-    auto dir = [&](int g, float (&uu)[DP4]) {
-#pragma unroll
-        for (int c = 0; c < DP4 / 4; ++c) {
-            const float4 v = *reinterpret_cast<const float4*>(uS + g * DP4 + 4 * c);
-            uu[4 * c] = v.x;
-            uu[4 * c + 1] = v.y;
-            uu[4 * c + 2] = v.z;
-            uu[4 * c + 3] = v.w;
-        }
-    };
-
-    // ---- pass A: every key of every direction counted in its histogram ------------------------
-    for (int i = tid; i < n; i += 2 * WNT) {
-        const int i2 = i + WNT;
-        const bool two = i2 < n;
-        float xa[DP4], xb[DP4];
-        rows(i, xa, xb, two, i2);
-#pragma unroll
-        for (int g = 0; g < WPC; ++g) {
-            if (g < GA) {
-                float uu[DP4];
-                dir(g, uu);
-                const float sc = C.sc_y[g], of = C.off_y[g];
-                unsigned* Hg = hist + g * (WNB / 2);
-                h16_add(Hg, bucket_fma<WNB>(key_w<D>(uu, xa), sc, of));
-                if (two) h16_add(Hg, bucket_fma<WNB>(key_w<D>(uu, xb), sc, of));
-            }
-        }
-    }
-    __syncthreads();
-
-    // ---- each warp: the runs of its direction ---------------------------------------------------
-    const int k1 = (n - 1) / 2, k2 = n / 2;
-    unsigned* H = hist + w * (WNB / 2);
-    int ba = 0, ca = 0, bb = 0, cb = 0, cnt0 = 0, c_lo1 = 0, cnt1 = 0, c_in = 0, fb = 0;
-    bool lr_set = false;
-    if (w < GA) {
-        wfind<true>(H, k1, k2, ba, ca, bb, cb);
-        cnt0 = cb + h16_get(H, bb) - ca;
-        fb = cnt0 > WCAP0 ? 1 : 0;
-        int c2 = 0, dl2 = OFF, dw2 = 0;
-        const int npos_guess = (n & 1) ? (n - 1) / 2 : n / 2;
-        if (ap && npos_guess > 0) {
-            const int base = n - npos_guess;
-            int b3, c3, b4, c4;
-            wfind<true>(H, base + (npos_guess - 1) / 2, base + npos_guess / 2, b3, c3, b4, c4);
-            c_lo1 = c3;
-            cnt1 = c4 + h16_get(H, b4) - c3;
-            if (cnt1 > WCAP1) fb = 1;
-            c2 = 2 * b3 + (b4 - b3);
-            dl2 = 0;
-            dw2 = b4 - b3;
-        } else if (!ap && !fb) {
-            wprefix(H);
-            // smallest s with more than k2 keys in the buckets [ba - s, bb + s] (the count grows with s and
-            // reaches n at s = WNB - 1): 32 lanes at steps of 64, then 64 values two per lane
-            auto win = [&](int s) {
-                const int hi = bb + s < WNB - 1 ? bb + s : WNB - 1;
-                return wP(H, hi) - wP(H, ba - s - 1);
-            };
-            const unsigned m1b = __ballot_sync(0xFFFFFFFFu, win(lane * 64) > k2);
-            const int f1 = m1b ? __ffs(m1b) - 1 : 32;
-            const int lo = f1 == 0 ? -1 : (f1 - 1) * 64;
-            const int sa = lo + 1 + 2 * lane, sb = sa + 1;
-            const unsigned ma = __ballot_sync(0xFFFFFFFFu, sa < WNB && win(sa) > k2);
-            const unsigned mb = __ballot_sync(0xFFFFFFFFu, sb < WNB && win(sb) > k2);
-            int ss = WNB;
-            if (ma) ss = lo + 1 + 2 * (__ffs(ma) - 1);
-            if (mb) ss = min(ss, lo + 2 + 2 * (__ffs(mb) - 1));
-            // the runs L, R of mad_runs (two buckets beyond the band on each side)
-            const int wd = bb - ba + 1;
-            const int L0 = ba - ss - wd - 2, L1 = ba - ss + wd + 3, R0 = bb + ss - wd - 3, R1 = bb + ss + wd + 2;
-            if (ss >= wd + 4 && L0 >= 1 && R1 <= WNB - 2) {
-                const int cl = (wP(H, L1) - wP(H, L0 - 1)) + (wP(H, R1) - wP(H, R0 - 1));
-                if (cl <= WCAP1) {
-                    cnt1 = cl;
-                    c_in = wP(H, R0 - 1) - wP(H, L1);
-                    c2 = ba + bb;
-                    dl2 = 2 * ss - wd - 7;
-                    dw2 = 4 * wd + 10;
-                    lr_set = true;
-                }
-            }
-        }
-        if (lane == 0) {
-            C.pa[w] = make_float4(C.sc_y[w], C.off_y[w], __int_as_float(fb ? OFF : ba), __int_as_float(bb - ba));
-            C.pb[w] = make_int4(c2, fb ? OFF : dl2, dw2, 0);
-            C.fill[w][0] = 0;
-            C.fill[w][1] = 0;
-        }
-    } else if (lane == 0) {
-        C.pa[w] = make_float4(0.0f, 0.0f, __int_as_float(OFF), __int_as_float(0));
-        C.pb[w] = make_int4(0, OFF, 0, 0);
-    }
-    __syncthreads();
-
-    // ---- gather pass: the keys of every direction's runs, with their point indices ---------------
-    for (int i = tid; i < n; i += 2 * WNT) {
-        const int i2 = i + WNT;
-        const bool two = i2 < n;
-        float xa[DP4], xb[DP4];
-        rows(i, xa, xb, two, i2);
-#pragma unroll
-        for (int g = 0; g < WPC; ++g) {
-            if (g < GA) {
-                float uu[DP4];
-                dir(g, uu);
-                const float4 pa = C.pa[g];
-                const int4 pb = C.pb[g];
-                const int bl0 = __float_as_int(pa.z), bw0 = __float_as_int(pa.w);
-                float* Bg = bufB + g * (WCAP0 + WCAP1);
-                int* Ig = bufI + g * (WCAP0 + WCAP1);
-                auto put = [&](float v, int idx) {
-                    const int b = bucket_fma<WNB>(v, pa.x, pa.y);
-                    if ((unsigned)(b - bl0) <= (unsigned)bw0) {
-                        const int pos = atomicAdd(&C.fill[g][0], 1);
-                        if (pos < WCAP0) {
-                            Bg[pos] = v;
-                            Ig[pos] = idx;
-                        }
-                    }
-                    if ((unsigned)(abs(2 * b - pb.x) - pb.y) <= (unsigned)pb.z) {
-                        const int pos = atomicAdd(&C.fill[g][1], 1);
-                        if (pos < WCAP1) {
-                            Bg[WCAP0 + pos] = v;
-                            Ig[WCAP0 + pos] = idx;
-                        }
-                    }
-                };
-                put(key_w<D>(uu, xa), i);
-                if (two) put(key_w<D>(uu, xb), i2);
-            }
-        }
-    }
-    __syncthreads();
-
-    // ---- each warp: ranks of its runs; D_P directions whose MAD runs did not hold (or overflowed) are
-    // flagged for the deviation passes ------------------------------------------------------------
-    const Grp<32> q{w, lane};
-    const KeysW<D> y{Dd.X32, uS + w * DP4, ldx};
-    float* B0 = bufB + w * (WCAP0 + WCAP1);
-    int* I0 = bufI + w * (WCAP0 + WCAP1);
-    float* B1 = B0 + WCAP0;
-    int* I1 = I0 + WCAP0;
-    float* tb = reinterpret_cast<float*>(H + NB2);   // pick scratch inside the histogram words
-    int* ti = reinterpret_cast<int*>(H + NB2 + 256);
-    constexpr int TC = 256;
-    const float qnan = __int_as_float(0x7FC00000);
-    float m1 = qnan, m2 = qnan, p1 = 0.f, p2 = 0.f, mf = 0.f, scd = 0.f;
-    int im1 = -1, im2 = -1, ip1 = -1, ip2 = -1, npos = 0;
-    bool dev = false;
-    if (w < GA && !fb) {
-        gpick_auto<32, TC>(q, B0, I0, cnt0, k1 - ca, k2 - ca, H, tb, ti, C, m1, m2, im1, im2);
-        if (ap) {
-            int c = 0;
-            for (int t = lane; t < cnt0; t += 32) c += (B0[t] <= m1);
-            const int nle = ca + gsum(q, c, C);
-            npos = n - nle;
-            if (npos > 0) {
-                const int s3 = nle + (npos - 1) / 2 - c_lo1, s4 = nle + npos / 2 - c_lo1;
-                if (s3 < 0 || s4 >= cnt1)
-                    fb = 2;   // the positive count differed from the guess
-                else
-                    gpick_auto<32, TC>(q, B1, I1, cnt1, s3, s4, H, tb, ti, C, p1, p2, ip1, ip2);
-            }
-        } else {
-            mf = __fmul_rn(__fadd_rn(m1, m2), 0.5f);
-            const bool ok = lr_set && mad_from_runs<32, TC>(q, B1, I1, cnt1, k1 - c_in, k2 - c_in, mf, H, tb, ti, C,
-                                                             p1, p2, ip1, ip2);
-            if (!ok) {
-                // |y - med| histogram over [0, 4 sigma_u] (edge bucket clamps) in the deviation passes
-                float dmax = Dd.cov ? 4.0f * C.scale[w] : 0.0f;
-                const float hard =
-                    __fmul_rn(__fadd_rn(Dd.rc, fabsf(mf - C.lo_b[w] - 0.5f * (float)WNB / C.sc_y[w])), 1.0001f);
-                if (!(dmax > 0.0f) || dmax > hard) dmax = hard;
-                if (!(dmax > 0.0f)) dmax = 1.0f;
-                scd = __fdiv_rn((float)WFBN, dmax);
-                dev = true;
-                for (int e = lane; e < WFBN; e += 32) H[e] = 0u;
-            }
-        }
-    }
-    if (lane == 0) {
-        C.dv[w] = make_float4(mf, scd, __int_as_float(dev ? 0 : OFF), __int_as_float(0));
-        if (dev) atomicAdd(&C.ndev, 1);
-    }
-    __syncthreads();
-
-    if (C.ndev > 0) {
-        // ---- deviation pass: |y - med| histograms of the flagged directions (32-bit, transposed) ----
-        for (int i = tid; i < n; i += 2 * WNT) {
-            const int i2 = i + WNT;
-            const bool two = i2 < n;
-            float xa[DP4], xb[DP4];
-            rows(i, xa, xb, two, i2);
-#pragma unroll 1
-            for (int g = 0; g < GA; ++g) {
-                const float4 dv = C.dv[g];
-                if (__float_as_int(dv.z) != 0) continue;
-                float uu[DP4];
-                dir(g, uu);
-                unsigned* Hg = hist + g * (WNB / 2);
-                atomicAdd(&Hg[hidx(bucket_fma<WFBN>(fabsf(__fsub_rn(key_w<D>(uu, xa), dv.x)), dv.y, 0.0f))], 1u);
-                if (two)
-                    atomicAdd(&Hg[hidx(bucket_fma<WFBN>(fabsf(__fsub_rn(key_w<D>(uu, xb), dv.x)), dv.y, 0.0f))], 1u);
-            }
-        }
-        __syncthreads();
-        int da = 0, dca = 0, db = 0, dcb = 0, cntd = 0;
-        if (dev) {
-            wfind<false>(H, k1, k2, da, dca, db, dcb);
-            cntd = dcb + (int)H[hidx(db)] - dca;
-            if (cntd > WCAP1) {
-                dev = false;
-                fb = 2;
-            }
-            if (lane == 0) {
-                C.dv[w].z = __int_as_float(dev ? da : OFF);
-                C.dv[w].w = __int_as_float(db - da);
-                C.fill[w][1] = 0;
-            }
-        }
-        __syncthreads();
-        // ---- deviation gather pass: the MAD runs of the flagged directions ----------------------------
-        for (int i = tid; i < n; i += 2 * WNT) {
-            const int i2 = i + WNT;
-            const bool two = i2 < n;
-            float xa[DP4], xb[DP4];
-            rows(i, xa, xb, two, i2);
-#pragma unroll 1
-            for (int g = 0; g < GA; ++g) {
-                const float4 dv = C.dv[g];
-                const int lo = __float_as_int(dv.z), wdt = __float_as_int(dv.w);
-                if (lo == OFF) continue;
-                float uu[DP4];
-                dir(g, uu);
-                float* Bg = bufB + g * (WCAP0 + WCAP1) + WCAP0;
-                int* Ig = bufI + g * (WCAP0 + WCAP1) + WCAP0;
-                auto put = [&](float v, int idx) {
-                    const float d1 = fabsf(__fsub_rn(v, dv.x));
-                    if ((unsigned)(bucket_fma<WFBN>(d1, dv.y, 0.0f) - lo) <= (unsigned)wdt) {
-                        const int pos = atomicAdd(&C.fill[g][1], 1);
-                        if (pos < WCAP1) {
-                            Bg[pos] = d1;
-                            Ig[pos] = idx;
-                        }
-                    }
-                };
-                put(key_w<D>(uu, xa), i);
-                if (two) put(key_w<D>(uu, xb), i2);
-            }
-        }
-        __syncthreads();
-        if (dev) gpick_auto<32, TC>(q, B1, I1, cntd, k1 - dca, k2 - dca, H, tb, ti, C, p1, p2, ip1, ip2);
-    }
-
-    if (w >= GA) return;   // no block barrier follows
-    const int64_t ro = S.roff + T.j0 + w;
-    close_warp<D>(q, y, C, H, B0, I0, n, ap, fb, m1, m2, im1, im2, p1, p2, ip1, ip2, npos, res + ro, err);
 }
 
 }  // namespace
@@ -2075,29 +1016,6 @@ __global__ void __launch_bounds__(KH_P) k_keys_halves(const TaskDev* __restrict_
         if (live[rr]) keys[(size_t)(r0 + rr) * npad + i] = key_halves<DP4>(Us[rr], xv);
 }
 
-size_t pdapw_smem_bytes(int d)
-{
-    const size_t dp4 = (size_t)((d + 3) & ~3);
-    return sizeof(float) * WPC * dp4 + sizeof(unsigned) * WPC * (WNB / 2) +
-           (sizeof(float) + sizeof(int)) * WPC * (WCAP0 + WCAP1);
-}
-
-bool pdapw_eligible(int64_t n, int d) { return d >= 1 && d <= 16 && n >= 1 && n <= PDAPW_MAX_N; }
-
-template <int D>
-static cudaError_t launch_w(const TaskDev* tasks, int ntasks, const SlotDev* slots, const DsDev* ds, const float* U,
-                            const double* yz, ResDev* res, int* err, cudaStream_t st)
-{
-    const size_t smem = pdapw_smem_bytes(D);
-    cudaError_t e = cudaFuncSetAttribute(k_pdapw<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return e;
-    }
-    k_pdapw<D><<<ntasks, WNT, smem, st>>>(tasks, slots, ds, U, res, err);
-    return cudaGetLastError();
-}
-
 template <int G, int DP4, bool STREAM>
 static cudaError_t launch_t(const TaskDev* tasks, int ntasks, size_t smem, const SlotDev* slots, const DsDev* ds,
                             const float* U, const double* yz, ResDev* res, int* err, const float* kin, cudaStream_t st)
@@ -2154,32 +1072,11 @@ static cudaError_t launch_select(const TaskDev* tasks, int ntasks, size_t smem, 
                                  int* err, cudaStream_t st, const float* kin)
 {
     if (smem > pdap_smem_limit()) return cudaErrorInvalidValue;
-    if (variant & PDAP_WARP) {
-        if (group < 1 || group > PDAPW_DIRS) return cudaErrorInvalidValue;
-        switch (variant & 0xFF) {
-        case 1: return launch_w<1>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 2: return launch_w<2>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 3: return launch_w<3>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 4: return launch_w<4>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 5: return launch_w<5>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 6: return launch_w<6>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 7: return launch_w<7>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 8: return launch_w<8>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 9: return launch_w<9>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 10: return launch_w<10>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 11: return launch_w<11>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 12: return launch_w<12>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 13: return launch_w<13>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 14: return launch_w<14>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 15: return launch_w<15>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        case 16: return launch_w<16>(tasks, ntasks, slots, ds, U, yz, res, err, st);
-        default: return cudaErrorInvalidValue;
-        }
-    }
+    if (variant & (PDAP_WARP | PDAP_KEYS)) return launch_sel(tasks, ntasks, group, variant, slots, ds, U, res, err, st, kin);
     const int dp4 = variant & ~PDAP_STREAM;
     if (variant & PDAP_STREAM) {
-        if (group != PDAP_STREAM_GROUP) return cudaErrorInvalidValue;
-        return launch_g<PDAP_STREAM_GROUP, true>(dp4, tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
+        if (group != PDAP_STREAM_GROUP || dp4 != 0) return cudaErrorInvalidValue;   // d <= 16 has k_select_x
+        return launch_t<PDAP_STREAM_GROUP, 0, true>(tasks, ntasks, smem, slots, ds, U, yz, res, err, nullptr, st);
     }
     switch (group) {
     case 1: return launch_g<1, false>(dp4, tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
@@ -2187,40 +1084,6 @@ static cudaError_t launch_select(const TaskDev* tasks, int ntasks, size_t smem, 
     case 4: return launch_g<4, false>(dp4, tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
     default: return cudaErrorInvalidValue;
     }
-}
-
-PdapShape pdap_shape(int n, int ldx, int m, int d, int group)
-{
-    PdapShape s{};
-    const int dp4 = pdap_dp4_class(d);
-    if (group == PDAP_WARP_GROUP && pdapw_eligible(n, d)) {
-        // one warp per direction, keys re-formed at every pass (taken when asked for: on the d = 10,
-        // n = 10,000 workload it runs 1.2x slower than two directions per CTA with resident keys); the
-        // query's m directions are spread evenly over its CTAs
-        const int ctas = (m + PDAPW_DIRS - 1) / PDAPW_DIRS;
-        s.group = (m + ctas - 1) / ctas;
-        s.variant = PDAP_WARP | d;
-        s.smem = pdapw_smem_bytes(d);
-        s.keys_gemm = false;
-        return s;
-    }
-    int G = (group == PDAP_WARP_GROUP || group == PDAP_STREAM_CHOICE) ? 0 : group;
-    if (G && (G > m || pdap_smem_bytes(n, G, ldx) > pdap_smem_limit())) G = 0;
-    if (!G && group != PDAP_STREAM_CHOICE) G = pdap_max_group(n, ldx, m, d, dp4 == 0, true);
-    if (G) {
-        s.group = G;
-        s.variant = dp4;
-        s.smem = pdap_smem_bytes(n, G, ldx);
-        s.keys_gemm = dp4 == 0;
-    } else {
-        s.group = PDAP_STREAM_GROUP;
-        s.variant = dp4 | PDAP_STREAM;
-        s.smem = pdap_smem_bytes(n, PDAP_STREAM_GROUP, ldx, true);
-        // the selection passes read keys formed once (k_keys, or k_keys_halves for d <= 16) instead of
-        // re-forming the dot products from X at every pass
-        s.keys_gemm = true;
-    }
-    return s;
 }
 
 size_t pdap_keys_bytes(int n, int group, int ntasks)

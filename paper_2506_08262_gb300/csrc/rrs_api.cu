@@ -279,10 +279,9 @@ rrs_status build_plan(const std::vector<ReqView>& reqs, Plan& P)
                 auto it = P.tune->find(std::make_tuple(D.n, D.ldx, m));
                 if (it != P.tune->end()) want = it->second;
             }
-            // resident keys when they fit shared memory, else keys formed once and read at every pass
-            const PdapShape sh = pdap_shape((int)D.n, D.ldx, m, D.d, want);
+            const PdapShape sh = pdap_shape((int)D.n, D.ldx, m, D.d, want, R.nq * (int64_t)m);
             G = sh.group;
-            // keys formed first by a keys kernel (d > 16, or keys outside shared memory): one list per
+            // keys formed first by a keys kernel (d > 16, or keys in device memory asked for): one list per
             // dataset, since a keys launch reads one X
             const int keys_ds = sh.keys_gemm ? dsidx[R.dset] : -1;
             for (size_t c : classes)
@@ -323,10 +322,14 @@ rrs_status build_plan(const std::vector<ReqView>& reqs, Plan& P)
             P.tot_d += D.d;
             P.max_ldx = std::max(P.max_ldx, D.ldx);
             for (int j0 = 0; j0 < m; j0 += 128) P.gen_tasks.push_back(TaskDev{s, j0, std::min(128, m - j0), 0});
-            if (R.kind != RRS_HALFSPACE) {
-                for (int j0 = 0; j0 < m; j0 += G) P.pd_tasks[cls].push_back(TaskDev{s, j0, std::min(G, m - j0), S.ds});
-            }
             P.argmin_list.push_back(s);
+        }
+        if (R.kind != RRS_HALFSPACE) {
+            // selection tasks: G consecutive (query, direction) rows of this request, across its queries
+            const int64_t rows = R.nq * (int64_t)m;
+            for (int64_t g = 0; g < rows; g += G)
+                P.pd_tasks[cls].push_back(TaskDev{s_first + (int)(g / m), (int)(g % m),
+                                                  (int)std::min<int64_t>(G, rows - g), dsidx[R.dset]});
         }
         if (R.kind == RRS_HALFSPACE && !tc) {
             // FP32 tasks: HD_ROWS consecutive (query, direction) rows of this request, across its queries
@@ -444,6 +447,30 @@ rrs_status upload_plan(rrs_ctx* ctx, Plan& P, cudaStream_t st)
     return RRS_OK;
 }
 
+// Enqueue the selection of the first `total` tasks of list c: one launch, or (keys in device memory) the keys and
+// the selection on them, one scratch-sized chunk at a time.
+rrs_status enqueue_selection(rrs_ctx* ctx, Plan& P, size_t c, int total, cudaStream_t st, bool capturing)
+{
+    const bool keys = P.pd_keys_ds[c] >= 0;
+    const int chunk = keys ? P.pd_keys_chunk[c] : total;
+    for (int t0 = 0; t0 < total; t0 += chunk) {
+        const int cnt = std::min(chunk, total - t0);
+        if (keys) {
+            StageTimer t(ctx, RRS_STAGE_KEYS, st, capturing);
+            CUDA_TRY(launch_pdap_keys(P.d_pd[c] + t0, cnt, P.pd_group[c], P.d_slots, P.d_ds, P.ds[P.pd_keys_ds[c]],
+                                      P.U, P.keys, st));
+            ctx->launches++;
+            ctx->stage_launches[RRS_STAGE_KEYS]++;
+        }
+        StageTimer t(ctx, RRS_STAGE_PDAP, st, capturing);
+        CUDA_TRY(launch_pdap(P.d_pd[c] + t0, cnt, P.pd_smem[c], P.pd_group[c], P.pd_variant[c], P.d_slots, P.d_ds,
+                             P.U, P.yz, P.res, ctx->d_err, st, keys ? P.keys : nullptr));
+        ctx->launches += PDAP_LAUNCH_KERNELS;
+        ctx->stage_launches[RRS_STAGE_PDAP]++;
+    }
+    return RRS_OK;
+}
+
 // Enqueue the whole refinement pipeline of a plan.
 rrs_status enqueue_rounds(rrs_ctx* ctx, Plan& P, cudaStream_t st, bool capturing = false)
 {
@@ -479,31 +506,8 @@ rrs_status enqueue_rounds(rrs_ctx* ctx, Plan& P, cudaStream_t st, bool capturing
             ctx->launches++;
         }
         for (size_t c = 0; c < P.pd_tasks.size(); ++c) {
-            if (P.n_pd[c][l] <= 0) continue;
-            if (P.pd_keys_ds[c] < 0) {
-                StageTimer t(ctx, RRS_STAGE_PDAP, st, capturing);
-                CUDA_TRY(launch_pdap(P.d_pd[c], P.n_pd[c][l], P.pd_smem[c], P.pd_group[c], P.pd_variant[c], P.d_slots,
-                                     P.d_ds, P.U, P.yz, P.res, ctx->d_err, st));
-                ctx->launches += PDAP_LAUNCH_KERNELS;
-                ctx->stage_launches[RRS_STAGE_PDAP]++;
-                continue;
-            }
-            // keys by the tiled GEMM, then the selection on them, one scratch-sized chunk at a time
-            const int total = P.n_pd[c][l], chunk = P.pd_keys_chunk[c];
-            for (int t0 = 0; t0 < total; t0 += chunk) {
-                const int cnt = std::min(chunk, total - t0);
-                {
-                    StageTimer t(ctx, RRS_STAGE_KEYS, st, capturing);
-                    CUDA_TRY(launch_pdap_keys(P.d_pd[c] + t0, cnt, P.pd_group[c], P.d_slots, P.d_ds,
-                                              P.ds[P.pd_keys_ds[c]], P.U, P.keys, st));
-                }
-                StageTimer t(ctx, RRS_STAGE_PDAP, st, capturing);
-                CUDA_TRY(launch_pdap(P.d_pd[c] + t0, cnt, P.pd_smem[c], P.pd_group[c], P.pd_variant[c], P.d_slots,
-                                     P.d_ds, P.U, P.yz, P.res, ctx->d_err, st, P.keys));
-                ctx->launches += 1 + PDAP_LAUNCH_KERNELS;
-                ctx->stage_launches[RRS_STAGE_KEYS]++;
-                ctx->stage_launches[RRS_STAGE_PDAP]++;
-            }
+            const rrs_status s = enqueue_selection(ctx, P, c, P.n_pd[c][l], st, capturing);
+            if (s != RRS_OK) return s;
         }
         if (P.n_arg[l] > 0) {
             StageTimer t(ctx, RRS_STAGE_ARGMIN, st, capturing);
@@ -615,9 +619,8 @@ rrs_status rrs_register_dataset(rrs_ctx* ctx, const void* X, int64_t n, int32_t 
                  bn = sizeof(float) * n;
     const bool want_cov = d <= RRS_COV_MAX_D;
     const size_t bmom = sizeof(float) * ((size_t)d + (want_cov ? (size_t)d * d : 0) + 1);
-    // the rows again in 32-row tiles for the selection kernels' projection pass (d <= 16: the kernels that
-    // hold directions in registers), which streams X once per CTA and is bound by the cache lines its loads touch
-    const size_t bt = d <= 16 ? sizeof(float) * tile_rows_floats(n, D.ldx) : 0;
+    // the data again as columns for the selection kernels that re-form keys from X (d <= 16)
+    const size_t bt = d <= 16 ? sizeof(float) * columns_floats(n, d) : 0;
     D.bytes = b32 + bt + b64 + bn + bmom;
     if (!budget_ok(ctx, D.bytes)) return fail(RRS_ERR_BUDGET, "dataset needs %zu bytes", D.bytes);
     void* staged = nullptr;
@@ -636,7 +639,7 @@ rrs_status rrs_register_dataset(rrs_ctx* ctx, const void* X, int64_t n, int32_t 
     if (e == cudaSuccess) e = cudaMemset(ctx->d_err, 0, sizeof(int));
     if (e == cudaSuccess) e = launch_convert_dataset(src, dtype, n, d, D.ldx, D.X32, D.X64, D.xnorm, ctx->d_err, st);
     if (e == cudaSuccess && D.Xt) {
-        e = launch_tile_rows(D.X32, n, D.ldx, D.Xt, st);
+        e = launch_columns(D.X32, n, d, D.ldx, D.Xt, st);
         ctx->launches++;
     }
     int bad = 0;
@@ -1018,11 +1021,10 @@ rrs_status rrs_debug_round_depths(rrs_ctx* ctx, int64_t dataset_id, const void* 
                 CUDA_TRY(launch_hd_simt(P.d_hd, (int)P.hd_tasks.size(), P.max_ldx, 0, P.d_slots, P.d_ds, P.U, P.yz,
                                         P.z64, P.res, band, ctx->d_err, st));
         } else {
-            for (size_t c = 0; c < P.pd_tasks.size(); ++c)
-                if (!P.pd_tasks[c].empty())
-                    CUDA_TRY(launch_pdap(P.d_pd[c], (int)P.pd_tasks[c].size(), P.pd_smem[c], P.pd_group[c],
-                                         P.pd_variant[c], P.d_slots, P.d_ds, P.U,
-                                         P.yz, P.res, ctx->d_err, st));
+            for (size_t c = 0; c < P.pd_tasks.size(); ++c) {
+                s = enqueue_selection(ctx, P, c, (int)P.pd_tasks[c].size(), st, true);
+                if (s != RRS_OK) return s;
+            }
         }
         ctx->launches += 4;
         trace("debug_round_depths: depth kernels enqueued");
@@ -1110,7 +1112,7 @@ rrs_status rrs_autotune(rrs_ctx* ctx, int64_t dataset_id, int32_t kind, int32_t 
     const std::vector<int> cands = hd ? std::vector<int>{256, 128}
                                       : std::vector<int>{1, 2, 4, PDAP_WARP_GROUP, PDAP_STREAM_CHOICE};
     for (int G : cands) {
-        if (!hd && (G == PDAP_WARP_GROUP ? !pdapw_eligible(D.n, D.d)
+        if (!hd && (G == PDAP_WARP_GROUP ? !pdap_x_eligible(D.d)
                                          : (G != PDAP_STREAM_CHOICE &&
                                             (G > m || pdap_smem_bytes((int)D.n, G, D.ldx) > pdap_smem_limit()))))
             continue;

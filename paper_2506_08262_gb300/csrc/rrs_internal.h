@@ -13,10 +13,8 @@ namespace rrs {
 // A resident dataset, as the kernels see it.
 struct DsDev {
     const float* X32;      // n x ldx FP32 rows, zero padded
-    // Xt: the FP32 rows again, for the selection kernels' projection pass (d <= 16), or nullptr.  Rows come in
-    // tiles of 32 (the last one zero padded); within a tile, 16-byte chunk c of its 32 rows is contiguous:
-    // float4 index ((i / 32) * (ldx / 4) + c) * 32 + i % 32.  A warp reading chunk c of 32 consecutive rows
-    // then reads 512 contiguous bytes (4 cache lines) where padded rows spread it over all 12 lines of d = 10.
+    // Xt: the FP32 data again as columns, for the selection kernels (d <= 16), or nullptr: dim l of point i at
+    // l * roundup32(n) + i, zero beyond n, so that a warp's lanes read consecutive points side by side.
     const float* Xt;
     const double* X64;     // n x d FP64 rows, or nullptr if the data came in FP32
     const float* xnorm;    // n Euclidean row norms, rounded up
@@ -116,12 +114,15 @@ constexpr int HD_ROWS = 64;
 cudaError_t launch_hd_simt(const TaskDev* tasks, int ntasks, int max_ldx, int64_t split_n, const SlotDev* slots, const DsDev* ds,
                            const float* U, const double* yz, const double* z64, ResDev* res, int64_t* band_out,
                            int* err, cudaStream_t st);
-// group: directions per CTA (1, 2 or 4, from pdap_shape); variant: pdap_shape's kernel variant (the key
-// arithmetic class pdap_dp4_class(d), plus PDAP_STREAM), shared by every task
+// group: directions per task and variant: the kernel, both from pdap_shape and shared by every task.  Where a
+// request's queries lie in consecutive slots a task may run from one query into the next, as for halfspace.
 // yz: the FP64 y_z = u'z of every direction (the direction generator's output), used for the depth.
 // Launches the selection kernel, which writes the points holding the order statistics into the result cells,
 // then k_pdap_finish, which forms the depths from FP64 projections of those points: PDAP_LAUNCH_KERNELS kernels.
 constexpr int PDAP_LAUNCH_KERNELS = 2;
+// its selection kernel for the variants PDAP_WARP and PDAP_KEYS (pdap_select.cu)
+cudaError_t launch_sel(const TaskDev* tasks, int ntasks, int group, int variant, const SlotDev* slots, const DsDev* ds,
+                       const float* U, ResDev* res, int* err, cudaStream_t st, const float* kin);
 cudaError_t launch_pdap(const TaskDev* tasks, int ntasks, size_t smem, int group, int variant, const SlotDev* slots,
                         const DsDev* ds, const float* U, const double* yz, ResDev* res, int* err, cudaStream_t st,
                         const float* kin = nullptr);
@@ -151,9 +152,9 @@ cudaError_t launch_debug_dirs(uint64_t seed, int q, int round0, int m, int d, fl
                               float* U, cudaStream_t st);
 cudaError_t launch_convert_dataset(const void* X, int dtype, int64_t n, int d, int ldx, float* X32,
                                    double* X64, float* xnorm, int* bad, cudaStream_t st);
-// DsDev::Xt from the padded rows X32 (Xt holds tile_rows_floats(n, ldx) floats)
-size_t tile_rows_floats(int64_t n, int ldx);
-cudaError_t launch_tile_rows(const float* X32, int64_t n, int ldx, float* Xt, cudaStream_t st);
+// DsDev::Xt from the padded rows X32 (Xt holds columns_floats(n, d) floats)
+size_t columns_floats(int64_t n, int d);
+cudaError_t launch_columns(const float* X32, int64_t n, int d, int ldx, float* Xt, cudaStream_t st);
 // mean, covariance (d <= RRS_COV_MAX_D) and radius about the mean of the FP32 rows; rc_out is a device float
 cudaError_t launch_moments(const float* X32, int64_t n, int d, int ldx, float* center, float* cov, float* rc_out,
                            cudaStream_t st);
@@ -163,33 +164,33 @@ size_t pdap_smem_limit();
 // preferred resident G; 0: keys outside shared memory (when allow_stream, or when none fits)
 int pdap_max_group(int n, int ldx, int m, int d, bool keys_in = false, bool allow_stream = false);
 
-// Selection-kernel variant bit: the keys are not held in shared memory (n beyond what shared memory holds
-// for one direction); every pass reads them from k_keys output in global memory when given (kin), else
-// recomputes them from X.  Such launches take PDAP_STREAM_GROUP directions per CTA.
+// Selection-kernel variant bit: no keys in shared memory, every pass recomputes them from X (the allocation-free
+// entry point with d > 16 where they do not fit).  Such launches take PDAP_STREAM_GROUP directions per CTA.
 constexpr int PDAP_STREAM = 0x100;
 // Largest n the selection kernels take: point indices and the padded key count (n rounded up to 4) are int.
 constexpr int64_t PDAP_MAX_N = 0x7FFFFFC0;
 constexpr int PDAP_STREAM_GROUP = 2;
-// Selection-kernel variant bit: one warp per direction, up to PDAPW_DIRS directions per CTA, keys re-formed
-// from X at every pass (d <= 16, n <= PDAPW_MAX_N: 16-bit bucket counters); the low byte holds d.  Asking
-// pdap_shape for group PDAP_WARP_GROUP selects it where it applies.
+// Selection-kernel variant bit: one warp per direction, keys re-formed from X at both passes (d <= 16); the low
+// byte holds d, bits 16 up the logarithm of the bucket count.  The default for d <= 16.
 constexpr int PDAP_WARP = 0x200;
-constexpr int PDAPW_DIRS = 12;
-constexpr int64_t PDAPW_MAX_N = 12288;
 constexpr int PDAP_WARP_GROUP = RRS_SELECT_WARP;
-// pdap_shape group asking for the keys outside shared memory (formed once per round, read at every pass)
+// Selection-kernel variant bit: keys formed once in device memory (launch_pdap_keys) and read at both passes, one
+// block per direction; bits 16 up hold the logarithm of the bucket count.  The default for d > 16.
+constexpr int PDAP_KEYS = 0x400;
+constexpr int PDAP_KEYS_GROUP = 8;
+// pdap_shape group asking for it
 constexpr int PDAP_STREAM_CHOICE = RRS_SELECT_STREAM;
-size_t pdapw_smem_bytes(int d);
-bool pdapw_eligible(int64_t n, int d);
+inline bool pdap_x_eligible(int d) { return d >= 1 && d <= 16; }
 struct PdapShape {
     int group;        // directions per CTA
-    int variant;      // pdap_dp4_class(d), plus PDAP_STREAM; or PDAP_WARP | d
+    int variant;      // pdap_dp4_class(d); or PDAP_WARP | d | log2 nb << 16; or PDAP_KEYS | log2 nb << 16
     size_t smem;      // dynamic shared memory per CTA
     bool keys_gemm;   // keys formed first by launch_pdap_keys
 };
-// Launch shape for a dataset (n rows, d dims, row stride ldx) and m directions per query; group > 0 asks for
-// that many resident directions per CTA (taken when it fits), 0 picks by the shared-memory heuristic.
-PdapShape pdap_shape(int n, int ldx, int m, int d, int group = 0);
+// Launch shape for a dataset (n rows, d dims, row stride ldx) and m directions per query.  group: 0 for the default,
+// 1, 2 or 4 for that many directions per CTA with resident keys (taken when they fit), PDAP_WARP_GROUP or
+// PDAP_STREAM_CHOICE.  rows: (query, direction) rows of the launch, 0 when unknown.
+PdapShape pdap_shape(int n, int ldx, int m, int d, int group = 0, int64_t rows = 0);
 
 // tensor-core path (hd_tc.cu)
 cudaError_t launch_build_bf16_planes(const float* X32, int64_t n, int d, int ldx, int kp, uint16_t* Xbf,

@@ -202,10 +202,15 @@ extern "C" rrs_status rrs_depth_noalloc(const void* X, int64_t n, int32_t d, int
     size_t pd_smem = 0;
     if (kind != RRS_HALFSPACE) {
         if (n > PDAP_MAX_N) return noalloc_fail(RRS_ERR_UNSUPPORTED, "n too large");
-        // keys formed inside the selection kernel (no k_keys scratch here): resident when they fit
-        // shared memory, else recomputed at every pass
-        int Gr = pdap_max_group((int)n, ldx, m, d);
-        if (Gr) {
+        // keys formed inside the selection kernel (no scratch for them here): re-formed from X for d <= 16; for
+        // larger d resident when they fit shared memory, else recomputed at every pass
+        if (pdap_x_eligible(d)) {
+            const PdapShape sh = pdap_shape((int)n, ldx, m, d, PDAP_WARP_GROUP, n_queries * (int64_t)m);
+            const int ctas = (m + sh.group - 1) / sh.group;
+            G = (m + ctas - 1) / ctas;   // a query's directions spread evenly over its CTAs
+            pd_variant = sh.variant;
+            pd_smem = sh.smem;
+        } else if (int Gr = pdap_max_group((int)n, ldx, m, d)) {
             G = Gr;
             pd_variant = pdap_dp4_class(d);
             pd_smem = pdap_smem_bytes((int)n, G, ldx);

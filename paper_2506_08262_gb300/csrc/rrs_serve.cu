@@ -422,7 +422,7 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
             PdapShape sh{};
             size_t cls = 0;
             if (R->kind != RRS_HALFSPACE) {
-                sh = pdap_shape((int)D.n, D.ldx, R->m, D.d);
+                sh = pdap_shape((int)D.n, D.ldx, R->m, D.d, 0, (int64_t)pick[ai].size() * R->m);
                 for (size_t c : classes)
                     if (sh.smem <= c) {
                         cls = c;
@@ -430,6 +430,8 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
                     }
             }
             const int G = sh.group;
+            // slots of a request need not be adjacent: tasks stay within a slot, its directions spread evenly
+            const int gper = G ? (R->m + ((R->m + G - 1) / G) - 1) / ((R->m + G - 1) / G) : 0;
             const int hper = (R->m + ((R->m + 63) / 64) - 1) / ((R->m + 63) / 64);
             const int row = S->ds_index[R->dataset];
             const bool use_tc = R->kind == RRS_HALFSPACE && S->precision == RRS_PREC_SPLIT_BF16X3 && D.kp > 0;
@@ -449,7 +451,7 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
                     auto& v = pd[key];
                     size_t& need = pd_need[key];
                     need = std::max(need, sh.smem);
-                    for (int j0 = 0; j0 < R->m; j0 += G) v.push_back(TaskDev{slot, j0, std::min(G, R->m - j0), row});
+                    for (int j0 = 0; j0 < R->m; j0 += gper) v.push_back(TaskDev{slot, j0, std::min(gper, R->m - j0), row});
                 }
                 arg.push_back(slot);
             }
