@@ -1102,13 +1102,23 @@ PdapShape pdap_shape(int n, int ldx, int m, int d, int group, int64_t rows)
         }
         group = 0;
     }
+    // a few directions on a long array: one per SM, all of a CTA's threads on it in every step, keys resident
+    // (n = 10,000, d = 5, 100 directions: 645 us per call against 672 with k_select_x, 682 with k_select;
+    // n = 2,000: 600 against 584, so short arrays stay with k_select_x)
+    if (group == 0 && dp4 && n > 4000 && rows > 0 && rows <= 2 * 152 && pdap_smem_bytes(n, 1, ldx) <= pdap_smem_limit()) {
+        s.group = 1;
+        s.variant = dp4;
+        s.smem = pdap_smem_bytes(n, 1, ldx);
+        s.keys_gemm = false;
+        return s;
+    }
     if (pdap_x_eligible(d) && group != PDAP_STREAM_CHOICE) {
         // keys re-formed from X: as many directions per CTA as its warps and shared memory take; fewer where the
         // request's rows would leave SMs without a CTA
         int G = SX_G;
         while (G > 1 && sel_smem(nb, G, d) > SX_SMEM) --G;
         const int64_t per_sm = (rows + 151) / 152;
-        if (rows > 0 && per_sm < G) G = per_sm <= 1 ? 1 : (per_sm <= 4 ? std::min(G, 4) : G);
+        if (rows > 0 && per_sm < G) G = per_sm <= 2 ? 1 : (per_sm <= 4 ? std::min(G, 4) : G);
         s.group = G;
         s.variant = PDAP_WARP | d | (lg << 16);
         s.smem = sel_smem(nb, G, d);

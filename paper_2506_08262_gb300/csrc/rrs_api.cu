@@ -210,6 +210,20 @@ rrs_status validate_params(int32_t kind, int32_t k, int32_t r, double alpha, int
     return RRS_OK;
 }
 
+// Keys scratch: one chunk of the largest keys list at a time, at most `limit` bytes (one task at least).
+void size_keys(Plan& P, size_t limit)
+{
+    P.keys_floats = 0;
+    for (size_t c = 0; c < P.pd_tasks.size(); ++c) {
+        if (P.pd_keys_ds[c] < 0 || P.pd_tasks[c].empty()) continue;
+        const int n = (int)P.ds[P.pd_keys_ds[c]].n;
+        const size_t per = pdap_keys_bytes(n, P.pd_group[c], 1);
+        const int chunk = (int)std::max<size_t>(1, std::min<size_t>(P.pd_tasks[c].size(), limit / per));
+        P.pd_keys_chunk[c] = chunk;
+        P.keys_floats = std::max(P.keys_floats, pdap_keys_bytes(n, P.pd_group[c], chunk) / sizeof(float));
+    }
+}
+
 // Build the launch plan for a set of requests (requests sorted by r, descending).
 rrs_status build_plan(const std::vector<ReqView>& reqs, Plan& P)
 {
@@ -387,16 +401,7 @@ rrs_status build_plan(const std::vector<ReqView>& reqs, Plan& P)
     for (auto& g : P.tc) prefix(g.tasks, g.n);
     P.n_pd.resize(P.pd_tasks.size());
     for (size_t c = 0; c < P.pd_tasks.size(); ++c) prefix(P.pd_tasks[c], P.n_pd[c]);
-    // keys scratch: one chunk of the largest keys list at a time, at most KEYS_SCRATCH_BYTES
-    constexpr size_t KEYS_SCRATCH_BYTES = 256u << 20;
-    for (size_t c = 0; c < P.pd_tasks.size(); ++c) {
-        if (P.pd_keys_ds[c] < 0 || P.pd_tasks[c].empty()) continue;
-        const int n = (int)P.ds[P.pd_keys_ds[c]].n;
-        const size_t per = pdap_keys_bytes(n, P.pd_group[c], 1);
-        const int chunk = (int)std::max<size_t>(1, std::min<size_t>(P.pd_tasks[c].size(), KEYS_SCRATCH_BYTES / per));
-        P.pd_keys_chunk[c] = chunk;
-        P.keys_floats = std::max(P.keys_floats, pdap_keys_bytes(n, P.pd_group[c], chunk) / sizeof(float));
-    }
+    size_keys(P, KEYS_SCRATCH_BYTES);
     P.n_arg.assign(P.rmax, 0);
     for (int l = 0; l < P.rmax; ++l) {
         int c = 0;
@@ -425,6 +430,19 @@ size_t carve_plan(Plan& P, Carve& C)
     P.res = C.take<ResDev>(P.tot_m);
     P.keys = P.keys_floats ? C.take<float>(P.keys_floats) : nullptr;
     return C.off;
+}
+
+// Workspace bytes of a plan; the smaller keys scratch where the larger one would exceed the context's budget.
+size_t plan_bytes(rrs_ctx* ctx, Plan& P)
+{
+    Carve sizing;
+    size_t bytes = carve_plan(P, sizing);
+    if (!budget_ok(ctx, bytes) && P.keys_floats) {
+        size_keys(P, KEYS_SCRATCH_MIN);
+        Carve again;
+        bytes = carve_plan(P, again);
+    }
+    return bytes;
 }
 
 // Upload the plan's host tables (slots, tasks) into the carved workspace.
@@ -733,8 +751,7 @@ static rrs_status run_requests(rrs_ctx* ctx, std::vector<ReqView>& reqs, cudaStr
     rrs_status s = build_plan(reqs, P);
     if (s != RRS_OK) return s;
     if (P.slots.empty()) return RRS_OK;
-    Carve sizing;
-    const size_t bytes = carve_plan(P, sizing);
+    const size_t bytes = plan_bytes(ctx, P);
     if (!budget_ok(ctx, bytes)) return fail(RRS_ERR_BUDGET, "call workspace needs %zu bytes", bytes);
     void* ws = nullptr;
     CUDA_TRY(cudaMallocAsync(&ws, bytes, st));
@@ -898,8 +915,7 @@ rrs_status rrs_depth_batched(rrs_ctx* ctx, const rrs_request* reqs, int32_t n_re
     P.tc_tune = &ctx->tc_tune;
     rrs_status s = build_plan(views, P);
     if (s != RRS_OK) return s;
-    Carve sizing;
-    const size_t bytes = carve_plan(P, sizing);
+    const size_t bytes = plan_bytes(ctx, P);
     if (!budget_ok(ctx, bytes)) return fail(RRS_ERR_BUDGET, "batched workspace needs %zu bytes", bytes);
     rrs_ctx::GraphEntry G;
     G.key = key;
@@ -993,8 +1009,7 @@ rrs_status rrs_debug_round_depths(rrs_ctx* ctx, int64_t dataset_id, const void* 
     Plan P;
     s = build_plan(reqs, P);
     if (s != RRS_OK) return s;
-    Carve sizing;
-    const size_t bytes = carve_plan(P, sizing) + sizeof(int64_t) * n_queries + 512;
+    const size_t bytes = plan_bytes(ctx, P) + sizeof(int64_t) * n_queries + 512;
     void* ws = nullptr;
     CUDA_TRY(cudaMalloc(&ws, bytes));
     Carve C;

@@ -131,6 +131,11 @@ cudaError_t launch_pdap(const TaskDev* tasks, int ntasks, size_t smem, int group
 // a tiled FP32 GEMM for d > 16 (where forming the keys inside the selection kernel re-reads X for every
 // G directions), two half chains per key for d <= 16 (used when the keys do not fit shared memory)
 size_t pdap_keys_bytes(int n, int group, int ntasks);
+// Bytes of selection keys formed at a time (one chunk of tasks: a keys launch, then the selection on them).  A chunk's
+// launches end in waves that are partly empty, so chunks are large: n = 100,000 at d = 100 took 117 / 89 / 74 / 66 ms
+// with 64 / 128 / 256 / 512 MB.  Where the context's budget has no room for KEYS_SCRATCH_BYTES the plan takes
+// KEYS_SCRATCH_MIN.
+constexpr size_t KEYS_SCRATCH_BYTES = (size_t)1 << 30, KEYS_SCRATCH_MIN = (size_t)256 << 20;
 cudaError_t launch_pdap_keys(const TaskDev* tasks, int ntasks, int group, const SlotDev* slots, const DsDev* ds,
                              const DsDev& ds_host, const float* U, float* keys, cudaStream_t st);
 int pdap_dp4_class(int d);

@@ -121,7 +121,7 @@ struct rrs_server {
     int ds_cap = 0;
     char* d_tab = nullptr;      // per-step tables (tasks, lists, new slots)
     size_t tab_bytes = 0;
-    float* d_keys = nullptr;    // selection keys formed by k_keys for d > 16 (at most KEYS_SCRATCH_BYTES)
+    float* d_keys = nullptr;    // selection keys formed by k_keys for d > 16, one chunk at a time
     size_t keys_bytes = 0;
     // host
     std::vector<int32_t> free_slots;
@@ -497,10 +497,10 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
                 continue;
             }
             // d > 16: keys by the tiled GEMM, then the selection on them, one scratch-sized chunk at a time
-            constexpr size_t KEYS_SCRATCH_BYTES = 256u << 20;
+            const size_t scratch = S->ctx->budget ? KEYS_SCRATCH_MIN : KEYS_SCRATCH_BYTES;
             const int n = (int)S->ds_host[krow].n;
             const size_t per = pdap_keys_bytes(n, G, 1);
-            const int chunk = (int)std::max<size_t>(1, std::min<size_t>(cnt_all, KEYS_SCRATCH_BYTES / per));
+            const int chunk = (int)std::max<size_t>(1, std::min<size_t>(cnt_all, scratch / per));
             const size_t need_b = pdap_keys_bytes(n, G, chunk);
             if (need_b > S->keys_bytes) {
                 if (S->d_keys) S_TRY(cudaFreeAsync(S->d_keys, S->st));
