@@ -411,6 +411,7 @@ rrs_status build_plan(const std::vector<ReqView>& reqs, Plan& P)
     return RRS_OK;
 }
 
+// The tables that upload_plan copies come first, d_ds the first of them and d_arg the last.
 size_t carve_plan(Plan& P, Carve& C)
 {
     P.d_ds = C.take<DsDev>(P.ds.size());
@@ -445,23 +446,27 @@ size_t plan_bytes(rrs_ctx* ctx, Plan& P)
     return bytes;
 }
 
-// Upload the plan's host tables (slots, tasks) into the carved workspace.
+// Upload the plan's host tables (datasets, slots, tasks) into the carved workspace: they are its first arrays, side by
+// side, so one copy of a host image of them serves (a copy of its own for each table costs more than a short kernel).
 rrs_status upload_plan(rrs_ctx* ctx, Plan& P, cudaStream_t st)
 {
     (void)ctx;
-    auto up = [&](void* dst, const void* src, size_t bytes) -> cudaError_t {
-        if (!bytes) return cudaSuccess;
-        return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+    char* base = (char*)P.d_ds;
+    const size_t total = (char*)P.d_arg - base + P.argmin_list.size() * sizeof(int32_t);
+    std::unique_ptr<char[]> image(new char[total]);
+    auto put = [&](void* dst, const void* src, size_t bytes) {
+        if (bytes) memcpy(image.get() + ((char*)dst - base), src, bytes);
     };
-    CUDA_TRY(up(P.d_ds, P.ds.data(), P.ds.size() * sizeof(DsDev)));
-    CUDA_TRY(up(P.d_slots, P.slots.data(), P.slots.size() * sizeof(SlotDev)));
-    CUDA_TRY(up(P.d_gen, P.gen_tasks.data(), P.gen_tasks.size() * sizeof(TaskDev)));
-    CUDA_TRY(up(P.d_hd, P.hd_tasks.data(), P.hd_tasks.size() * sizeof(TaskDev)));
-    for (auto& g : P.tc) CUDA_TRY(up(g.d, g.tasks.data(), g.tasks.size() * sizeof(TaskDev)));
-    if (P.d_maps) CUDA_TRY(up(P.d_maps, P.maps.data(), P.maps.size() * sizeof(CUtensorMap)));
+    put(P.d_ds, P.ds.data(), P.ds.size() * sizeof(DsDev));
+    put(P.d_slots, P.slots.data(), P.slots.size() * sizeof(SlotDev));
+    put(P.d_gen, P.gen_tasks.data(), P.gen_tasks.size() * sizeof(TaskDev));
+    put(P.d_hd, P.hd_tasks.data(), P.hd_tasks.size() * sizeof(TaskDev));
+    for (auto& g : P.tc) put(g.d, g.tasks.data(), g.tasks.size() * sizeof(TaskDev));
+    if (P.d_maps) put(P.d_maps, P.maps.data(), P.maps.size() * sizeof(CUtensorMap));
     for (size_t c = 0; c < P.pd_tasks.size(); ++c)
-        CUDA_TRY(up(P.d_pd[c], P.pd_tasks[c].data(), P.pd_tasks[c].size() * sizeof(TaskDev)));
-    CUDA_TRY(up(P.d_arg, P.argmin_list.data(), P.argmin_list.size() * sizeof(int32_t)));
+        put(P.d_pd[c], P.pd_tasks[c].data(), P.pd_tasks[c].size() * sizeof(TaskDev));
+    put(P.d_arg, P.argmin_list.data(), P.argmin_list.size() * sizeof(int32_t));
+    CUDA_TRY(cudaMemcpyAsync(base, image.get(), total, cudaMemcpyHostToDevice, st));   // pageable: staged on return
     return RRS_OK;
 }
 
@@ -539,9 +544,9 @@ rrs_status enqueue_rounds(rrs_ctx* ctx, Plan& P, cudaStream_t st, bool capturing
 
 rrs_status check_device_errors(rrs_ctx* ctx, cudaStream_t st)
 {
-    int h = 0;
-    CUDA_TRY(cudaMemcpyAsync(&h, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaMemcpyAsync(ctx->h_flag, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
+    const int h = *ctx->h_flag;
     if (h) {
         cudaMemsetAsync(ctx->d_err, 0, sizeof(int), st);
         cudaStreamSynchronize(st);
@@ -588,7 +593,25 @@ rrs_status rrs_create(rrs_ctx** out, int32_t device, uint64_t hbm_budget_bytes)
     c->device = device;
     c->budget = hbm_budget_bytes;
     CUDA_TRY(cudaMalloc(&c->d_err, sizeof(int)));
-    CUDA_TRY(cudaMemset(c->d_err, 0, sizeof(int)));
+    cudaError_t e = cudaMemset(c->d_err, 0, sizeof(int));
+    if (e == cudaSuccess) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        e = cudaMemPoolCreate(&c->pool, &props);
+    }
+    if (e == cudaSuccess) {
+        uint64_t keep = hbm_budget_bytes ? 0 : rrs_ctx::POOL_KEEP;
+        e = cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+    if (e == cudaSuccess) e = cudaMallocHost(&c->h_flag, sizeof(int));
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        if (c->pool) cudaMemPoolDestroy(c->pool);
+        cudaFree(c->d_err);
+        return fail(RRS_ERR_CUDA, "context set-up failed: %s", cudaGetErrorString(e));
+    }
     *out = c.release();
     return RRS_OK;
 }
@@ -616,6 +639,8 @@ rrs_status rrs_destroy(rrs_ctx* ctx)
     }
     for (auto e : ctx->event_pool) cudaEventDestroy(e);
     cudaFree(ctx->d_err);
+    cudaMemPoolDestroy(ctx->pool);
+    cudaFreeHost(ctx->h_flag);
     delete ctx;
     return RRS_OK;
 }
@@ -742,7 +767,10 @@ static void drop_graphs(rrs_ctx* ctx)
     cudaGetLastError();
 }
 
-static rrs_status run_requests(rrs_ctx* ctx, std::vector<ReqView>& reqs, cudaStream_t st, int force_group = 0)
+// verdict: called once the plan is built and uploaded, before any of its kernels is enqueued; a failure ends the call.
+// rrs_depth waits there for its input check, which runs while the host builds the plan.
+template <class F>
+static rrs_status run_requests(rrs_ctx* ctx, std::vector<ReqView>& reqs, cudaStream_t st, int force_group, F verdict)
 {
     Plan P;
     P.tune = &ctx->pd_tune;
@@ -750,16 +778,17 @@ static rrs_status run_requests(rrs_ctx* ctx, std::vector<ReqView>& reqs, cudaStr
     P.force_group = force_group;
     rrs_status s = build_plan(reqs, P);
     if (s != RRS_OK) return s;
-    if (P.slots.empty()) return RRS_OK;
+    if (P.slots.empty()) return verdict();
     const size_t bytes = plan_bytes(ctx, P);
     if (!budget_ok(ctx, bytes)) return fail(RRS_ERR_BUDGET, "call workspace needs %zu bytes", bytes);
     void* ws = nullptr;
-    CUDA_TRY(cudaMallocAsync(&ws, bytes, st));
+    CUDA_TRY(cudaMallocFromPoolAsync(&ws, bytes, ctx->pool, st));
     Carve C;
     C.base = (char*)ws;
     C.cap = bytes;
     carve_plan(P, C);
     s = upload_plan(ctx, P, st);
+    if (s == RRS_OK) s = verdict();
     if (s == RRS_OK) s = enqueue_rounds(ctx, P, st);
     cudaFreeAsync(ws, st);
     return s;
@@ -798,7 +827,7 @@ rrs_status rrs_depth(rrs_ctx* ctx, int64_t dataset_id, const void* Z, int64_t n_
                  ob_choice = 4 * n_queries * r;
     const size_t obytes = ob_depth + ob_count + ob_best + ob_choice + 64;
     if (!z_on_device) {
-        CUDA_TRY(cudaMallocAsync(&zdev, zbytes, st));
+        CUDA_TRY(cudaMallocFromPoolAsync(&zdev, zbytes, ctx->pool, st));
         CUDA_TRY(cudaMemcpyAsync(zdev, Z, zbytes, cudaMemcpyHostToDevice, st));
     }
     const void* zsrc = z_on_device ? Z : zdev;
@@ -823,25 +852,30 @@ rrs_status rrs_depth(rrs_ctx* ctx, int64_t dataset_id, const void* Z, int64_t n_
         R.best_out = best_out;
         R.choice_out = round_choice_out;
     } else {
-        CUDA_TRY(cudaMallocAsync((void**)&outdev, obytes, st));
+        CUDA_TRY(cudaMallocFromPoolAsync((void**)&outdev, obytes, ctx->pool, st));
         R.depth_out = (double*)outdev;
         R.count_out = (int64_t*)(outdev + ob_depth);
         R.best_out = (int32_t*)(outdev + ob_depth + ob_count);
         R.choice_out = (int32_t*)(outdev + ob_depth + ob_count + ob_best);
     }
-    // the finiteness check must pass before any compute is trusted: read it now
-    int bad = 0;
-    CUDA_TRY(cudaMemcpyAsync(&bad, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    if (bad) {
-        cudaMemsetAsync(ctx->d_err, 0, sizeof(int), st);
-        if (zdev) cudaFreeAsync(zdev, st);
-        if (outdev) cudaFreeAsync(outdev, st);
-        cudaStreamSynchronize(st);
-        return fail(RRS_ERR_INVALID_ARG, "Z holds a non-finite value or one of magnitude >= 2^64");
-    }
+    CUDA_TRY(cudaMemcpyAsync(ctx->h_flag, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     std::vector<ReqView> reqs{R};
-    s = run_requests(ctx, reqs, st);
+    // the finiteness check must pass before any compute is trusted; it runs while the plan is built
+    bool waited = false;
+    auto verdict = [&]() -> rrs_status {
+        waited = true;
+        CUDA_TRY(cudaStreamSynchronize(st));
+        if (!*ctx->h_flag) return RRS_OK;
+        cudaMemsetAsync(ctx->d_err, 0, sizeof(int), st);
+        return fail(RRS_ERR_INVALID_ARG, "Z holds a non-finite value or one of magnitude >= 2^64");
+    };
+    s = run_requests(ctx, reqs, st, 0, verdict);
+    // a plan that could not be built must not hide a bad query batch, which is reported first
+    if (s != RRS_OK && !waited) {
+        const std::string why = rrs_last_error();
+        const rrs_status v = verdict();
+        s = v != RRS_OK ? v : fail(s, "%s", why.c_str());
+    }
     if (s == RRS_OK && !out_on_device) {
         CUDA_TRY(cudaMemcpyAsync(depth_out, R.depth_out, ob_depth, cudaMemcpyDeviceToHost, st));
         if (count_out) CUDA_TRY(cudaMemcpyAsync(count_out, R.count_out, ob_count, cudaMemcpyDeviceToHost, st));
@@ -899,7 +933,7 @@ rrs_status rrs_depth_batched(rrs_ctx* ctx, const rrs_request* reqs, int32_t n_re
         views.push_back(R);
     }
     if (views.empty()) return RRS_OK;
-    if (!use_graph) return run_requests(ctx, views, st);
+    if (!use_graph) return run_requests(ctx, views, st, 0, [] { return RRS_OK; });
 
     // graph path: identical descriptors replay a captured launch sequence
     std::vector<char> key((const char*)reqs, (const char*)reqs + sizeof(rrs_request) * n_requests);
@@ -1147,7 +1181,7 @@ rrs_status rrs_autotune(rrs_ctx* ctx, int64_t dataset_id, int32_t kind, int32_t 
         for (int rep = 0; rep < 3; ++rep) {
             std::vector<ReqView> reqs{R};
             CUDA_TRY(cudaEventRecord(a, 0));
-            s = run_requests(ctx, reqs, 0, hd ? 0 : G);
+            s = run_requests(ctx, reqs, 0, hd ? 0 : G, [] { return RRS_OK; });
             if (s != RRS_OK) break;
             CUDA_TRY(cudaEventRecord(b, 0));
             CUDA_TRY(cudaEventSynchronize(b));

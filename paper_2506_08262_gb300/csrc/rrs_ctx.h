@@ -40,6 +40,12 @@ struct rrs_ctx {
     std::map<int64_t, rrs::Dataset> datasets;
     uint64_t launches = 0;
     int* d_err = nullptr;
+    // pool of the per-call workspaces: the context's own, so that memory stays mapped from one call to the next (the
+    // device's default pool gives it back at every synchronisation, and mapping it again costs more than a short
+    // call), up to POOL_KEEP bytes; a context with a budget keeps nothing.  Given back by rrs_destroy.
+    static constexpr uint64_t POOL_KEEP = (uint64_t)2 << 30;
+    cudaMemPool_t pool = nullptr;
+    int* h_flag = nullptr;   // pinned: device-side flags read back without a staged copy
     std::mutex mu;
     // cached captured graphs of batched calls (keyed by the request bytes)
     struct GraphEntry {

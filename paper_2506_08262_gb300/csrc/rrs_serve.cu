@@ -197,7 +197,7 @@ rrs_status step_table(rrs_server* S, size_t bytes)
     if (bytes <= S->tab_bytes) return RRS_OK;
     if (S->d_tab) S_TRY(cudaFreeAsync(S->d_tab, S->st));
     const size_t nb = std::max(bytes, S->tab_bytes * 2);
-    S_TRY(cudaMallocAsync((void**)&S->d_tab, nb, S->st));
+    S_TRY(cudaMallocFromPoolAsync((void**)&S->d_tab, nb, S->ctx->pool, S->st));
     S->tab_bytes = nb;
     return RRS_OK;
 }
@@ -215,8 +215,8 @@ rrs_status admit(rrs_server* S)
         const DsDev& D = S->ds_host[row];
         const size_t esz = R->dtype == RRS_F32 ? 4 : 8;
         const size_t zbytes = esz * (size_t)R->nq * D.d;
-        S_TRY(cudaMallocAsync(&R->zdev, zbytes, S->st));
-        S_TRY(cudaMallocAsync((void**)&R->ddev, sizeof(double) * R->nq, S->st));
+        S_TRY(cudaMallocFromPoolAsync(&R->zdev, zbytes, S->ctx->pool, S->st));
+        S_TRY(cudaMallocFromPoolAsync((void**)&R->ddev, sizeof(double) * R->nq, S->ctx->pool, S->st));
         S_TRY(cudaMemcpyAsync(R->zdev, R->Zhost, zbytes, cudaMemcpyHostToDevice, S->st));
         // cost weight of a pair: the tensor-core halfspace path runs about ten times as many pairs per second
         // as the FP32 and selection paths (measured)
@@ -255,7 +255,7 @@ rrs_status admit(rrs_server* S)
     if (news.empty()) return RRS_OK;
     const size_t b1 = sizeof(SlotDev) * news.size(), b2 = sizeof(int32_t) * idx.size();
     char* tmp = nullptr;
-    S_TRY(cudaMallocAsync((void**)&tmp, b1 + 256 + b2, S->st));
+    S_TRY(cudaMallocFromPoolAsync((void**)&tmp, b1 + 256 + b2, S->ctx->pool, S->st));
     S_TRY(cudaMemcpyAsync(tmp, news.data(), b1, cudaMemcpyHostToDevice, S->st));
     S_TRY(cudaMemcpyAsync(tmp + b1 + 256 - (b1 % 256), idx.data(), b2, cudaMemcpyHostToDevice, S->st));
     const int cnt = (int)news.size();
@@ -505,7 +505,7 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
             if (need_b > S->keys_bytes) {
                 if (S->d_keys) S_TRY(cudaFreeAsync(S->d_keys, S->st));
                 S->d_keys = nullptr;
-                S_TRY(cudaMallocAsync((void**)&S->d_keys, need_b, S->st));
+                S_TRY(cudaMallocFromPoolAsync((void**)&S->d_keys, need_b, S->ctx->pool, S->st));
                 S->keys_bytes = need_b;
             }
             for (int t0 = 0; t0 < cnt_all; t0 += chunk) {
