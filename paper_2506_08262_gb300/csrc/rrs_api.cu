@@ -156,6 +156,7 @@ struct Plan {
     // per round whatever the datasets: every task's CTA takes its dataset's tensor map from maps
     struct TcGroup {
         int kp = 0, bn = 0;   // K extent of the planes, points per tile
+        int64_t max_n = 0;    // largest n among its datasets
         std::vector<TaskDev> tasks;
         std::vector<int> n;   // active prefix per round
         TaskDev* d = nullptr;
@@ -381,6 +382,7 @@ rrs_status build_plan(const std::vector<ReqView>& reqs, Plan& P)
                 P.tc.back().bn = bn;
             }
             const int64_t rows = R.nq * (int64_t)m;
+            P.tc[gi].max_n = std::max(P.tc[gi].max_n, D.n);
             for (int64_t g = 0; g < rows; g += 128)
                 P.tc[gi].tasks.push_back(
                     TaskDev{s_first + (int)(g / m), (int)(g % m), (int)std::min<int64_t>(128, rows - g), 0});
@@ -523,7 +525,7 @@ rrs_status enqueue_rounds(rrs_ctx* ctx, Plan& P, cudaStream_t st, bool capturing
         for (auto& g : P.tc) {
             if (g.n[l] <= 0) continue;
             StageTimer t(ctx, RRS_STAGE_HD_TC, st, capturing);
-            CUDA_TRY(launch_hd_tc(g.d, g.n[l], g.kp, g.bn, P.d_slots, P.d_ds, P.d_maps, P.U, P.yz, P.z64, P.res,
+            CUDA_TRY(launch_hd_tc(g.d, g.n[l], g.kp, g.bn, g.max_n, P.d_slots, P.d_ds, P.d_maps, P.U, P.yz, P.z64, P.res,
                                   nullptr, ctx->d_err, st));
             ctx->stage_launches[RRS_STAGE_HD_TC]++;
             ctx->launches++;
@@ -1064,7 +1066,7 @@ rrs_status rrs_debug_round_depths(rrs_ctx* ctx, int64_t dataset_id, const void* 
         trace("debug_round_depths: y_z done");
         if (kind == RRS_HALFSPACE) {
             if (precision == RRS_PREC_SPLIT_BF16X3)
-                CUDA_TRY(launch_hd_tc(P.tc[0].d, (int)P.tc[0].tasks.size(), P.tc[0].kp, P.tc[0].bn, P.d_slots, P.d_ds, P.d_maps, P.U, P.yz,
+                CUDA_TRY(launch_hd_tc(P.tc[0].d, (int)P.tc[0].tasks.size(), P.tc[0].kp, P.tc[0].bn, 0, P.d_slots, P.d_ds, P.d_maps, P.U, P.yz,
                                       P.z64, P.res, band, ctx->d_err, st));
             else
                 CUDA_TRY(launch_hd_simt(P.d_hd, (int)P.hd_tasks.size(), P.max_ldx, 0, P.d_slots, P.d_ds, P.U, P.yz,

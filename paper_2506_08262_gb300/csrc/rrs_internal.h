@@ -111,6 +111,7 @@ cudaError_t launch_gen(const TaskDev* tasks, int ntasks, const SlotDev* slots, c
 // split_n: the largest n among the tasks' datasets, which lets a launch of few tasks split the points over more
 // CTAs (the result cells must then be zero, as launch_gen leaves them); 0: no split
 constexpr int HD_ROWS = 64;
+constexpr int HD_PART_SHIFT = 48;   // bits of a count in a result cell shared by the parts of a split (n < 2^48)
 cudaError_t launch_hd_simt(const TaskDev* tasks, int ntasks, int max_ldx, int64_t split_n, const SlotDev* slots, const DsDev* ds,
                            const float* U, const double* yz, const double* z64, ResDev* res, int64_t* band_out,
                            int* err, cudaStream_t st);
@@ -209,7 +210,8 @@ cudaError_t encode_tc_map(const DsDev& ds_host, int bn, CUtensorMap* out);
 // tasks of up to 128 (query, direction) rows each, of any datasets whose planes have K extent kp and whose maps
 // were encoded for tiles of bn points; maps[ds] is the tensor map of dataset row ds of ds_dev (device memory,
 // 64-byte aligned)
-cudaError_t launch_hd_tc(const TaskDev* tasks, int ntasks, int kp, int bn, const SlotDev* slots,
+// split_n: as for launch_hd_simt
+cudaError_t launch_hd_tc(const TaskDev* tasks, int ntasks, int kp, int bn, int64_t split_n, const SlotDev* slots,
                          const DsDev* ds_dev, const CUtensorMap* maps, const float* U, const double* yz,
                          const double* z64, ResDev* res, int64_t* band_out, int* err, cudaStream_t st);
 bool hd_tc_supported(int d);

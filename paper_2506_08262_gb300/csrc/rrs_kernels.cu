@@ -364,7 +364,6 @@ constexpr int HD_NT = 128;
 constexpr int HD_TJ = HD_ROWS;   // rows (query, direction) per CTA
 constexpr int HD_PC = 256;       // points per chunk
 constexpr int HD_K = 16;         // dims per staging step
-constexpr int HD_PART_SHIFT = 48;   // bits of a count in a result cell shared by the parts of a split (n < 2^48)
 
 // Parts the points are split into.  Two CTAs share an SM, and a launch of few tasks leaves SMs empty or ends in a
 // wave that is nearly empty: below eight waves of tasks the points are split into as many parts as give about

@@ -409,6 +409,7 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
         int64_t hd_n = 0;   // largest n among the FP32 halfspace datasets of the step
         // (K extent of the planes, points per tile) -> tensor-core halfspace tasks
         std::map<std::pair<int, int>, std::vector<TaskDev>> tc;
+        std::map<std::pair<int, int>, int64_t> tc_n;   // their largest n
         // selection lists per (shared-memory class, G, kernel variant, dataset row for keys by k_keys or -1);
         // each launch requests the largest shared-memory need of its list
         std::map<std::tuple<size_t, int, int, int>, std::vector<TaskDev>> pd;
@@ -441,6 +442,8 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
                 if (use_tc) {
                     // slots of a request need not be adjacent: one task never crosses a slot
                     auto& v = tc[std::make_pair(D.kp, S->ds_bn[row])];
+                    int64_t& nmax = tc_n[std::make_pair(D.kp, S->ds_bn[row])];
+                    nmax = std::max(nmax, D.n);
                     for (int j0 = 0; j0 < R->m; j0 += 128) v.push_back(TaskDev{slot, j0, std::min(128, R->m - j0), 0});
                 } else if (R->kind == RRS_HALFSPACE) {
                     hd_n = std::max(hd_n, D.n);
@@ -484,7 +487,7 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
                              S->d_yz, S->d_z64, S->d_res, nullptr, S->ctx->d_err, S->st));
         for (auto& to : o_tc)
             S_TRY(launch_hd_tc((const TaskDev*)(T + to.first), (int)tc[to.second].size(), to.second.first,
-                               to.second.second, S->d_slots, S->d_ds, S->d_maps, S->d_U, S->d_yz, S->d_z64, S->d_res,
+                               to.second.second, tc_n[to.second], S->d_slots, S->d_ds, S->d_maps, S->d_U, S->d_yz, S->d_z64, S->d_res,
                                nullptr, S->ctx->d_err, S->st));
         size_t extra = 0;
         for (auto& po : o_pd) {

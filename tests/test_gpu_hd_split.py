@@ -28,3 +28,19 @@ def test_counts_equal_the_oracle(n, d, nq, k, r, dtype):
     assert np.array_equal(cnt.cpu().numpy(), ref["count"])
     assert np.array_equal(best.cpu().numpy(), ref["best"])
     assert np.array_equal(dep.cpu().numpy(), ref["depth"])
+
+
+# the tensor-core kernel's parts: at least 8 tiles of 256 (d <= 62) or 128 points
+@pytest.mark.parametrize("n", [2047, 4096, 4097, 9001, 20_001])
+@pytest.mark.parametrize("d,nq,k,r,dtype", [(3, 3, 63, 1, np.float32), (62, 4, 150, 2, np.float32),
+                                            (63, 2, 130, 2, np.float32), (100, 2, 65, 1, np.float64)])
+def test_tensor_core_counts_equal_the_oracle(n, d, nq, k, r, dtype):
+    X, Z = workloads.gaussian_cloud(12, n, d, nq, dtype=dtype)
+    Z[0] = X[n - 1]
+    with rrs.Context(0) as ctx:
+        did = ctx.register(torch.from_numpy(X).cuda())
+        dep, cnt, best = ctx.depth(did, torch.from_numpy(Z).cuda(), rrs.RRS_HALFSPACE, k, r, 0.5, seed=3,
+                                   precision=rrs.RRS_PREC_SPLIT_BF16X3)
+    ref = oracle.rrs(X, Z, oracle.HALFSPACE, k, r, 0.5, 3)
+    assert np.array_equal(cnt.cpu().numpy(), ref["count"])
+    assert np.array_equal(best.cpu().numpy(), ref["best"])
