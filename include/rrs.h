@@ -61,7 +61,8 @@ typedef int32_t rrs_status;
 /*
  * rrs_create - open a context on CUDA device `device`.
  *   hbm_budget_bytes: upper bound on the device memory the context may hold
- *   for datasets and per-call workspace; 0 means no bound.
+ *   for datasets and per-call workspace; 0 means no bound.  Without a bound the
+ *   context keeps up to 2 GB of workspace from one call to the next.
  *   *out receives the context.  Errors: INVALID_ARG (out NULL, bad device),
  *   CUDA.
  */
@@ -107,12 +108,12 @@ rrs_status rrs_free(rrs_ctx* ctx, int64_t dataset_id);
  *   Projection depths select the points holding the median / MAD / MAD_+ of
  *   the FP32 projections (exact order statistics of the FP32 keys, ties broken
  *   by point index) and form the depth from FP64 projections of those points
- *   and of z.  The keys are held in shared memory while two CTAs of two
- *   directions fit an SM (about n <= 10,000 for d <= 12); beyond that they are
- *   formed once per round in device memory (up to 256 MB of scratch, taken in
- *   chunks) and every selection pass reads them back, with the same
- *   arithmetic, so results do not depend on which form ran.  n is limited to
- *   2^31 - 64 for projection depths.
+ *   and of z.  For d <= 16 the keys are re-formed from the data at both passes
+ *   of the selection; for larger d they are formed once per round in device
+ *   memory (up to 1 GB of scratch, 256 MB where the context's budget has no room
+ *   for more, taken in chunks) and read back at both passes.  The arithmetic is
+ *   the same in every form, so results do not depend on which ran.  n is limited
+ *   to 2^31 - 64 for projection depths.
  * Outputs (each n_queries long, or n_queries*r for round_choice_out):
  *   depth_out[q]   final depth D_min (double).                      required
  *   count_out[q]   halfspace: min(#<=, #>=) at D_min, else -1.        optional
@@ -184,17 +185,14 @@ rrs_status rrs_depth_batched(rrs_ctx* ctx, const rrs_request* reqs, int32_t n_re
  * directions per round: 1, 2 or 4 directions per CTA with the keys held in
  * shared memory, RRS_SELECT_STREAM (keys formed once per round in device
  * memory and read at every pass), or RRS_SELECT_WARP (one warp per direction,
- * keys re-formed from X at every pass; d <= 16 and n <= 12,288).  Each
- * feasible choice is
+ * keys re-formed from X at every pass; d <= 16).  Each feasible choice is
  * timed on one round of probe queries (rows of the dataset, two per SM) and
  * the fastest is cached in the context; later rrs_depth / rrs_depth_batched
- * calls with the same (n, d, m) use it.  Without tuning: two or more
- * directions per CTA with resident keys where that fits two CTAs per SM,
- * else the streamed keys.  Results
+ * calls with the same (n, d, m) use it.  Without tuning: RRS_SELECT_WARP for
+ * d <= 16 (one resident direction per CTA where n > 4,000 and the request has
+ * at most two directions per SM), RRS_SELECT_STREAM for larger d.  Results
  * never depend on the choice.  *choice_out (optional) receives it (0 for
- * halfspace depth, which has nothing to tune, and 0 when no choice keeps the
- * keys in shared memory: they then live in device memory and the kernel runs
- * with a fixed shape).
+ * halfspace depth with one tile width).
  * Synchronous.  Errors: INVALID_ARG, NOT_FOUND, CUDA.
  */
 #define RRS_SELECT_WARP 64

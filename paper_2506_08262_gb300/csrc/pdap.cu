@@ -3,10 +3,13 @@
 // MAD_+) of the FP32 keys, whose points a second kernel (k_pdap_finish)
 // re-projects in FP64 to form the depth.
 //
-// One CTA handles G <= 4 directions of one query with the G*n keys resident in
-// shared memory, or, when n is beyond what shared memory holds, G = 2
-// directions whose keys stay outside: formed once by a keys kernel and read
-// from global memory at every pass, or (allocation-free entry point)
+// The default selection kernels are in pdap_select.cu; this file holds the kernel
+// with its keys in shared memory (k_pdap2), the keys kernels, the FP64 finish and
+// the launch of a selection.  k_pdap2 runs for a few directions on a long array
+// and where rrs_select_kernel or the autotuner ask for 1, 2 or 4 directions per CTA.
+//
+// One CTA handles G <= 4 directions with the G*n keys resident in shared memory,
+// or (allocation-free entry point, d > 16, n beyond what shared memory holds)
 // recomputed from X at every pass; the arithmetic is the same throughout, and
 // so are the values.  The whole CTA projects (pass A: every point on the G
 // directions, keys stored, each added to a 2048-bucket histogram over
