@@ -149,7 +149,7 @@ struct Plan {
     std::vector<int> n_gen, n_hd, n_arg;
     std::vector<std::vector<int>> n_pd;
     int rmax = 0;
-    int max_ldx = 4;
+    int max_ldx = 4, max_m = 0;
     int64_t hd_n = 0;   // largest n among the FP32 halfspace datasets
     int64_t tot_ldx = 0, tot_d = 0, tot_u = 0, tot_m = 0;
     // tensor-core halfspace tasks, one group per K extent of the planes (64 or 128), each group one launch
@@ -282,6 +282,7 @@ rrs_status build_plan(const std::vector<ReqView>& reqs, Plan& P)
         const ReqView& R = reqs[ri];
         const Dataset& D = *R.dset;
         const int m = (R.k + R.r - 1) / R.r;
+        P.max_m = std::max(P.max_m, m);
         int G = 0;
         int cls = -1;
         const bool tc = R.kind == RRS_HALFSPACE && R.precision == RRS_PREC_SPLIT_BF16X3;
@@ -500,6 +501,7 @@ rrs_status enqueue_selection(rrs_ctx* ctx, Plan& P, size_t c, int total, cudaStr
 rrs_status enqueue_rounds(rrs_ctx* ctx, Plan& P, cudaStream_t st, bool capturing = false)
 {
     const int64_t T = P.tot_ldx;
+    const bool fused = P.max_m <= NEXT_MAX_M;   // one generation task per slot: round end and next start in one launch
     {
         StageTimer t(ctx, RRS_STAGE_PREP, st, capturing);
         CUDA_TRY(launch_prep(P.d_slots, (int)P.slots.size(), P.d_ds, P.z32, P.z64, P.poles, st));
@@ -509,7 +511,7 @@ rrs_status enqueue_rounds(rrs_ctx* ctx, Plan& P, cudaStream_t st, bool capturing
     for (int l = 0; l < P.rmax; ++l) {
         float* cur = P.poles + (l & 1) * T;
         float* nxt = P.poles + ((l + 1) & 1) * T;
-        if (P.n_gen[l] > 0) {
+        if (P.n_gen[l] > 0 && (l == 0 || !fused)) {
             StageTimer t(ctx, RRS_STAGE_GEN, st, capturing);
             CUDA_TRY(launch_gen(P.d_gen, P.n_gen[l], P.d_slots, cur, P.z64, P.U, P.yz, P.res, l, P.max_ldx, st));
             ctx->launches++;
@@ -536,7 +538,10 @@ rrs_status enqueue_rounds(rrs_ctx* ctx, Plan& P, cudaStream_t st, bool capturing
         }
         if (P.n_arg[l] > 0) {
             StageTimer t(ctx, RRS_STAGE_ARGMIN, st, capturing);
-            CUDA_TRY(launch_argmin(P.d_slots, P.d_arg, P.n_arg[l], P.U, P.res, cur, nxt, l, 0, st));
+            if (fused)
+                CUDA_TRY(launch_next(P.d_slots, P.d_arg, P.n_arg[l], cur, nxt, P.z64, P.U, P.yz, P.res, l, P.max_ldx, st));
+            else
+                CUDA_TRY(launch_argmin(P.d_slots, P.d_arg, P.n_arg[l], P.U, P.res, cur, nxt, l, 0, st));
             ctx->launches++;
             ctx->stage_launches[RRS_STAGE_ARGMIN]++;
         }

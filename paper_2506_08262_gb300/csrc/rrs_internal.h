@@ -143,6 +143,10 @@ int pdap_dp4_class(int d);
 cudaError_t launch_argmin(SlotDev* slots, const int32_t* slot_list, int nlist, const float* U,
                           const ResDev* res, const float* poles_cur, float* poles_next, int round0,
                           int last_round, cudaStream_t st);
+// launch_argmin of round round0 and launch_gen of the next in one launch, for slots of at most NEXT_MAX_M directions
+constexpr int NEXT_MAX_M = 128;
+cudaError_t launch_next(SlotDev* slots, const int32_t* slot_list, int nlist, const float* poles_cur, float* poles_next,
+                        const double* z64, float* U, double* yz, ResDev* res, int round0, int max_ldx, cudaStream_t st);
 cudaError_t launch_yz_only(const TaskDev* tasks, int ntasks, const SlotDev* slots, const double* z64,
                            const float* U, double* yz, cudaStream_t st);
 cudaError_t launch_scatter_dirs(const SlotDev* slots, int nslots, int m, int d, const float* Uin, float* U,

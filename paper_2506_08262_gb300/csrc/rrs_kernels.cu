@@ -206,6 +206,43 @@ cudaError_t launch_prep(const SlotDev* slots, int nslots, const DsDev* ds, float
 constexpr int GEN_NT = 128, GEN_STRIDE = GEN_NT + 1;
 constexpr size_t GEN_STAGE_MAX = 96 * 1024;
 
+// The directions j0 .. j0 + nj - 1 of one query for round rnd around its pole, by a CTA of GEN_NT threads.
+__device__ __forceinline__ void gen_rows(const SlotDev& S, int j0, int nj, int rnd, const float* pole,
+                                         const double* __restrict__ z64, float* __restrict__ U,
+                                         double* __restrict__ yz, ResDev* __restrict__ res, int stage_d, float* gstage)
+{
+    const int jl = threadIdx.x, j = j0 + jl;
+    const float ap = alpha_power(S.alpha, rnd);
+    const double* z = z64 + S.zoff64;
+    // zero result cells: where the halfspace kernels split the points they add their counts there
+    if (jl < nj) res[S.roff + j] = ResDev{0.0, 0};
+    if (S.d > stage_d) {
+        if (jl >= nj) return;
+        float* u = U + S.uoff + (int64_t)j * S.ldx;
+        stream_direction(S.seed, (uint32_t)S.qctr, (uint32_t)rnd, (uint32_t)j, S.d, ap, pole, u, 1);
+        for (int l = S.d; l < S.ldx; ++l) u[l] = 0.0f;
+        double acc = 0.0;
+        for (int l = 0; l < S.d; ++l) acc = __fma_rn((double)u[l], z[l], acc);
+        yz[S.roff + j] = acc;
+        return;
+    }
+    if (jl < nj) {
+        float* u = gstage + jl;
+        stream_direction(S.seed, (uint32_t)S.qctr, (uint32_t)rnd, (uint32_t)j, S.d, ap, pole, u, GEN_STRIDE);
+        double acc = 0.0;
+        for (int l = 0; l < S.d; ++l) acc = __fma_rn((double)u[l * GEN_STRIDE], z[l], acc);
+        yz[S.roff + j] = acc;
+    }
+    __syncthreads();
+    // rows j0 .. j0 + nj - 1 of this query are contiguous in U
+    float* base = U + S.uoff + (int64_t)j0 * S.ldx;
+    const int ldx = S.ldx, total = nj * ldx;
+    for (int e = jl; e < total; e += GEN_NT) {
+        const int r = e / ldx, l = e - r * ldx;
+        base[e] = l < S.d ? gstage[l * GEN_STRIDE + r] : 0.0f;
+    }
+}
+
 __global__ void __launch_bounds__(GEN_NT) k_gen(const TaskDev* __restrict__ tasks, const SlotDev* __restrict__ slots,
                                                 const float* __restrict__ poles, const float* __restrict__ poles1,
                                                 const double* __restrict__ z64, float* __restrict__ U,
@@ -213,54 +250,117 @@ __global__ void __launch_bounds__(GEN_NT) k_gen(const TaskDev* __restrict__ task
 {
     extern __shared__ float gstage[];
     const TaskDev T = tasks[blockIdx.x];
-    const int jl = threadIdx.x;
     const SlotDev& S = slots[T.slot];
     // launch-wide round, or (round0 < 0) the slot's own round with its pole buffer by parity
     const int rnd = round0 >= 0 ? round0 : S.round;
     const float* pcur = round0 >= 0 ? poles : ((rnd & 1) ? poles1 : poles);
-    const int j = T.j0 + jl;
-    const float ap = alpha_power(S.alpha, rnd);
-    const double* z = z64 + S.zoff64;
-    // zero result cells: where the halfspace kernel splits the points it adds its counts there
-    if (jl < T.nj) res[S.roff + j] = ResDev{0.0, 0};
-    if (S.d > stage_d) {
-        if (jl >= T.nj) return;
-        float* u = U + S.uoff + (int64_t)j * S.ldx;
-        stream_direction(S.seed, (uint32_t)S.qctr, (uint32_t)rnd, (uint32_t)j, S.d, ap, pcur + S.zoff32, u, 1);
-        for (int l = S.d; l < S.ldx; ++l) u[l] = 0.0f;
-        double acc = 0.0;
-        for (int l = 0; l < S.d; ++l) acc = __fma_rn((double)u[l], z[l], acc);
-        yz[S.roff + j] = acc;
-        return;
+    gen_rows(S, T.j0, T.nj, rnd, pcur + S.zoff32, z64, U, yz, res, stage_d, gstage);
+}
+
+// The end of round round0 and the start of the next for slots of at most GEN_NT directions, one CTA per slot: the
+// round minimum and the pole update (k_argmin's rules), then, unless that was the slot's last round, its next
+// directions around the new pole (k_gen's).  One launch where two of them each cost a short call a launch gap per
+// round.
+__global__ void __launch_bounds__(GEN_NT) k_next(SlotDev* __restrict__ slots, const int32_t* __restrict__ slot_list,
+                                                 const float* __restrict__ pcur, float* __restrict__ pnext,
+                                                 const double* __restrict__ z64, float* __restrict__ U,
+                                                 double* __restrict__ yz, ResDev* __restrict__ res, int round0, int stage_d)
+{
+    extern __shared__ float gstage[];
+    __shared__ double sv[GEN_NT / 32];
+    __shared__ int64_t sc[GEN_NT / 32];
+    __shared__ int sj[GEN_NT / 32];
+    SlotDev& S = slots[slot_list[blockIdx.x]];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, m = S.m;
+    const bool hd = (S.kind == 0);
+    double bv = INFINITY;
+    int64_t bc = INT64_MAX;
+    int bj = INT32_MAX;
+    if (tid < m) {
+        const ResDev r = res[S.roff + tid];
+        if (hd ? (r.count < bc) : (r.depth < bv)) {
+            bv = r.depth;
+            bc = r.count;
+            bj = tid;
+        }
     }
-    if (jl < T.nj) {
-        float* u = gstage + jl;
-        stream_direction(S.seed, (uint32_t)S.qctr, (uint32_t)rnd, (uint32_t)j, S.d, ap, pcur + S.zoff32, u,
-                         GEN_STRIDE);
-        double acc = 0.0;
-        for (int l = 0; l < S.d; ++l) acc = __fma_rn((double)u[l * GEN_STRIDE], z[l], acc);
-        yz[S.roff + j] = acc;
+    auto merge = [&](double ov, int64_t oc, int oj) {
+        const bool better = hd ? (oc < bc || (oc == bc && oj < bj)) : (ov < bv || (ov == bv && oj < bj));
+        if (better) {
+            bv = ov;
+            bc = oc;
+            bj = oj;
+        }
+    };
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xFFFFFFFFu, bv, o);
+        const int64_t oc = __shfl_xor_sync(0xFFFFFFFFu, bc, o);
+        const int oj = __shfl_xor_sync(0xFFFFFFFFu, bj, o);
+        merge(ov, oc, oj);
     }
+    if (lane == 0) {
+        sv[w] = bv;
+        sc[w] = bc;
+        sj[w] = bj;
+    }
+    const int64_t cmin = S.cmin;
+    const double dmin = S.dmin;
     __syncthreads();
-    // rows j0 .. j0 + nj - 1 of this query are contiguous in U
-    float* base = U + S.uoff + (int64_t)T.j0 * S.ldx;
-    const int ldx = S.ldx, total = T.nj * ldx;
-    for (int e = jl; e < total; e += GEN_NT) {
-        const int r = e / ldx, l = e - r * ldx;
-        base[e] = l < S.d ? gstage[l * GEN_STRIDE + r] : 0.0f;
+#pragma unroll
+    for (int i = 0; i < GEN_NT / 32; ++i) merge(sv[i], sc[i], sj[i]);   // every thread gets the same minimum
+    const bool take = hd ? (bc < cmin) : (bv < dmin);
+    const float* src = take ? U + S.uoff + (int64_t)bj * S.ldx : pcur + S.zoff32;
+    for (int l = tid; l < S.ldx; l += GEN_NT) pnext[S.zoff32 + l] = src[l];
+    const bool last = round0 == S.r - 1;
+    if (tid == 0) {
+        const int best = take ? round0 * m + bj : S.best;
+        if (take) {
+            S.dmin = bv;
+            S.cmin = bc;
+            S.best = best;
+        }
+        if (S.choice_out) S.choice_out[round0] = take ? bj : -1;
+        if (last) {
+            if (S.depth_out) S.depth_out[0] = take ? bv : dmin;
+            if (S.count_out) S.count_out[0] = hd ? (take ? bc : cmin) : -1;
+            if (S.best_out) S.best_out[0] = best;
+        }
     }
+    if (last) return;
+    __syncthreads();   // the new pole is written, and the old directions are no longer read
+    gen_rows(S, 0, m, round0 + 1, pnext + S.zoff32, z64, U, yz, res, stage_d, gstage);
 }
 
 // directions of up to max_ldx dims are staged in shared memory (up to GEN_STAGE_MAX bytes)
+static int gen_stage_d(int max_ldx)
+{
+    const size_t per_dim = sizeof(float) * GEN_STRIDE;
+    return (size_t)max_ldx * per_dim > GEN_STAGE_MAX ? (int)(GEN_STAGE_MAX / per_dim) : max_ldx;
+}
+
+cudaError_t launch_next(SlotDev* slots, const int32_t* slot_list, int nlist, const float* poles_cur, float* poles_next,
+                        const double* z64, float* U, double* yz, ResDev* res, int round0, int max_ldx, cudaStream_t st)
+{
+    if (nlist <= 0) return cudaSuccess;
+    const int stage_d = gen_stage_d(max_ldx);
+    const size_t smem = (size_t)stage_d * sizeof(float) * GEN_STRIDE;
+    const cudaError_t e = cudaFuncSetAttribute(k_next, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e;
+    }
+    k_next<<<nlist, GEN_NT, smem, st>>>(slots, slot_list, poles_cur, poles_next, z64, U, yz, res, round0, stage_d);
+    return cudaGetLastError();
+}
+
 static cudaError_t gen_launch(const TaskDev* tasks, int ntasks, const SlotDev* slots, const float* p0,
                               const float* p1, const double* z64, float* U, double* yz, ResDev* res, int round0,
                               int max_ldx, cudaStream_t st)
 {
     if (ntasks <= 0) return cudaSuccess;
-    int stage_d = max_ldx;
-    const size_t per_dim = sizeof(float) * GEN_STRIDE;
-    if ((size_t)stage_d * per_dim > GEN_STAGE_MAX) stage_d = (int)(GEN_STAGE_MAX / per_dim);
-    const size_t smem = (size_t)stage_d * per_dim;
+    const int stage_d = gen_stage_d(max_ldx);
+    const size_t smem = (size_t)stage_d * sizeof(float) * GEN_STRIDE;
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(k_gen, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) {
