@@ -289,12 +289,16 @@ extern "C" rrs_status rrs_depth_noalloc(const void* X, int64_t n, int32_t d, int
     for (int l = 0; l < n_refinements; ++l) {
         float* cur = poles + (l & 1) * T;
         float* nxt = poles + ((l + 1) & 1) * T;
-        NA_TRY(launch_gen(gen, nq * gen_per, slots, cur, z64, U, yz, res, l, ldx, st));
+        if (l == 0 || m > NEXT_MAX_M)
+            NA_TRY(launch_gen(gen, nq * gen_per, slots, cur, z64, U, yz, res, l, ldx, st));
         if (kind == RRS_HALFSPACE)
             NA_TRY(launch_hd_simt(hd, nq * hd_per, ldx, n, slots, ds, U, yz, z64, res, nullptr, err + 1, st));
         else
             NA_TRY(launch_pdap(pd, nq * pd_per, pd_smem, G, pd_variant, slots, ds, U, yz, res, err + 1, st));
-        NA_TRY(launch_argmin(slots, arg, nq, U, res, cur, nxt, l, 0, st));
+        if (m <= NEXT_MAX_M)
+            NA_TRY(launch_next(slots, arg, nq, cur, nxt, z64, U, yz, res, l, ldx, st));
+        else
+            NA_TRY(launch_argmin(slots, arg, nq, U, res, cur, nxt, l, 0, st));
     }
     int flags = 0;
     NA_TRY(cudaMemcpyAsync(&flags, err + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
