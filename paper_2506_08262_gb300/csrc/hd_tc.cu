@@ -829,11 +829,9 @@ cudaError_t launch_hd_tc(const TaskDev* tasks, int ntasks, int kp, int bn, int64
     if (bn != tc_tile_n(kp, bn)) return cudaErrorInvalidValue;
     const size_t smem = tc_smem_bytes(kp, bn);
     auto kern = bn == 256 ? k_hd_tc<256> : k_hd_tc<128>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return e;
-    }
+    static SmemLimit limit[2];
+    const cudaError_t e = limit[bn == 256].raise(kern);
+    if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)ntasks, (unsigned)tc_parts(ntasks, split_n, bn));
     kern<<<grid, NTHREADS, smem, st>>>(maps, tasks, slots, ds_dev, U, yz, z64, res, band_out, err,
                                          band_gamma_tc(kp), tc_stages(kp, bn));

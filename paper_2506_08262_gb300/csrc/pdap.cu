@@ -1023,12 +1023,9 @@ template <int G, int DP4, bool STREAM>
 static cudaError_t launch_t(const TaskDev* tasks, int ntasks, size_t smem, const SlotDev* slots, const DsDev* ds,
                             const float* U, const double* yz, ResDev* res, int* err, const float* kin, cudaStream_t st)
 {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_pdap2<G, DP4, STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) {
-        cudaGetLastError();   // do not leave the failure pending for an unrelated later call
-        return e;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise(k_pdap2<G, DP4, STREAM>);
+    if (e != cudaSuccess) return e;
     k_pdap2<G, DP4, STREAM><<<ntasks, cta_threads<G>(), smem, st>>>(tasks, slots, ds, U, res, err, kin);
     return cudaGetLastError();
 }

@@ -1027,11 +1027,9 @@ cudaError_t launch_x(const TaskDev* tasks, int ntasks, int G, int nb, const Slot
                             const float* U, ResDev* res, int* err, cudaStream_t st)
 {
     const size_t smem = sel_smem(nb, G, D);
-    const cudaError_t e = cudaFuncSetAttribute(k_select_x<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return e;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise(k_select_x<D>);
+    if (e != cudaSuccess) return e;
     k_select_x<D><<<ntasks, SX_NT, smem, st>>>(tasks, slots, ds, U, res, err, nb, G);
     return cudaGetLastError();
 }
@@ -1041,11 +1039,9 @@ cudaError_t launch_k(const TaskDev* tasks, int ntasks, int G, int nb, const Slot
                             ResDev* res, int* err, const float* kin, cudaStream_t st)
 {
     const size_t smem = sel_smem(nb, 1, 0);
-    const cudaError_t e = cudaFuncSetAttribute(k_select<GS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return e;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise(k_select<GS>);
+    if (e != cudaSuccess) return e;
     k_select<GS><<<ntasks * G, GS, smem, st>>>(tasks, G, slots, ds, res, err, kin, nb);
     return cudaGetLastError();
 }

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/rrs.h"
 
 namespace rrs {
@@ -95,6 +97,32 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn encode_fn();
 __host__ __device__ float band_coef_ff(int d);   // bound coefficient of the compensated FP32 re-check (tensor-core path)
+
+// Dynamic shared memory a kernel may ask for: raised once per device to the most its static memory leaves, by the first
+// launch there.  The limit belongs to the kernel, not to a launch: one that set its own size on every call could lower
+// it between another host thread's setting and that thread's launch.  One object per kernel.
+class SmemLimit {
+    std::atomic<uint64_t> done_{0};   // devices 0 .. 63 whose limit is raised
+
+public:
+    template <class K>
+    cudaError_t raise(K* kernel)
+    {
+        int dev = 0, most = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess && dev < 64 && (done_.load(std::memory_order_acquire) >> dev & 1)) return e;
+        cudaFuncAttributes a{};
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, kernel);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes);
+        if (e != cudaSuccess)
+            cudaGetLastError();   // do not leave the failure pending for an unrelated later call
+        else if (dev < 64)
+            done_.fetch_or(1ull << dev, std::memory_order_release);
+        return e;
+    }
+};
 
 // Set the text that rrs_last_error() returns on this thread (rrs_api.cu).
 void set_last_error(const char* msg);

@@ -345,11 +345,9 @@ cudaError_t launch_next(SlotDev* slots, const int32_t* slot_list, int nlist, con
     if (nlist <= 0) return cudaSuccess;
     const int stage_d = gen_stage_d(max_ldx);
     const size_t smem = (size_t)stage_d * sizeof(float) * GEN_STRIDE;
-    const cudaError_t e = cudaFuncSetAttribute(k_next, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return e;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise(k_next);
+    if (e != cudaSuccess) return e;
     k_next<<<nlist, GEN_NT, smem, st>>>(slots, slot_list, poles_cur, poles_next, z64, U, yz, res, round0, stage_d);
     return cudaGetLastError();
 }
@@ -361,13 +359,9 @@ static cudaError_t gen_launch(const TaskDev* tasks, int ntasks, const SlotDev* s
     if (ntasks <= 0) return cudaSuccess;
     const int stage_d = gen_stage_d(max_ldx);
     const size_t smem = (size_t)stage_d * sizeof(float) * GEN_STRIDE;
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_gen, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return e;
-        }
-    }
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise(k_gen);
+    if (e != cudaSuccess) return e;
     k_gen<<<ntasks, GEN_NT, smem, st>>>(tasks, slots, p0, p1, z64, U, yz, res, round0, stage_d);
     return cudaGetLastError();
 }
@@ -733,11 +727,9 @@ cudaError_t launch_hd_simt(const TaskDev* tasks, int ntasks, int max_ldx, int64_
 {
     if (ntasks <= 0) return cudaSuccess;
     const size_t smem = sizeof(float) * ((size_t)HD_TJ * max_ldx + 2 * HD_K * HD_PC + 2 * HD_PC);
-    const cudaError_t e = cudaFuncSetAttribute(k_hd_simt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return e;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise(k_hd_simt);
+    if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)ntasks, (unsigned)hd_parts(ntasks, split_n));
     k_hd_simt<<<grid, HD_NT, smem, st>>>(tasks, slots, ds, U, yz, z64, res, band_out, err);
     return cudaGetLastError();
