@@ -1091,6 +1091,14 @@ size_t pdap_keys_bytes(int n, int group, int ntasks)
     return sizeof(float) * (size_t)ntasks * group * (((size_t)n + 3) & ~(size_t)3);
 }
 
+int pdap_keys_chunk(int n, int d, int group, int64_t ntasks, size_t bytes)
+{
+    // rows of one keys launch: its grid's y extent, each block a tile of KH_D or KT_D rows
+    const int64_t rows = (int64_t)65535 * (pdap_dp4_class(d) ? KH_D : KT_D);
+    const int64_t most = std::min<int64_t>(rows / group, (int64_t)(bytes / pdap_keys_bytes(n, group, 1)));
+    return (int)std::max<int64_t>(1, std::min(ntasks, most));
+}
+
 cudaError_t launch_pdap_keys(const TaskDev* tasks, int ntasks, int group, const SlotDev* slots, const DsDev* ds,
                              const DsDev& ds_host, const float* U, float* keys, cudaStream_t st)
 {

@@ -217,9 +217,9 @@ void size_keys(Plan& P, size_t limit)
     P.keys_floats = 0;
     for (size_t c = 0; c < P.pd_tasks.size(); ++c) {
         if (P.pd_keys_ds[c] < 0 || P.pd_tasks[c].empty()) continue;
-        const int n = (int)P.ds[P.pd_keys_ds[c]].n;
-        const size_t per = pdap_keys_bytes(n, P.pd_group[c], 1);
-        const int chunk = (int)std::max<size_t>(1, std::min<size_t>(P.pd_tasks[c].size(), limit / per));
+        const DsDev& D = P.ds[P.pd_keys_ds[c]];
+        const int n = (int)D.n;
+        const int chunk = pdap_keys_chunk(n, D.d, P.pd_group[c], (int64_t)P.pd_tasks[c].size(), limit);
         P.pd_keys_chunk[c] = chunk;
         P.keys_floats = std::max(P.keys_floats, pdap_keys_bytes(n, P.pd_group[c], chunk) / sizeof(float));
     }

@@ -165,6 +165,8 @@ size_t pdap_keys_bytes(int n, int group, int ntasks);
 // with 64 / 128 / 256 / 512 MB.  Where the context's budget has no room for KEYS_SCRATCH_BYTES the plan takes
 // KEYS_SCRATCH_MIN.
 constexpr size_t KEYS_SCRATCH_BYTES = (size_t)1 << 30, KEYS_SCRATCH_MIN = (size_t)256 << 20;
+// Tasks of one keys launch: at most `bytes` of keys and what its grid holds, one at least.
+int pdap_keys_chunk(int n, int d, int group, int64_t ntasks, size_t bytes);
 cudaError_t launch_pdap_keys(const TaskDev* tasks, int ntasks, int group, const SlotDev* slots, const DsDev* ds,
                              const DsDev& ds_host, const float* U, float* keys, cudaStream_t st);
 int pdap_dp4_class(int d);

@@ -502,8 +502,7 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
             // d > 16: keys by the tiled GEMM, then the selection on them, one scratch-sized chunk at a time
             const size_t scratch = S->ctx->budget ? KEYS_SCRATCH_MIN : KEYS_SCRATCH_BYTES;
             const int n = (int)S->ds_host[krow].n;
-            const size_t per = pdap_keys_bytes(n, G, 1);
-            const int chunk = (int)std::max<size_t>(1, std::min<size_t>(cnt_all, scratch / per));
+            const int chunk = pdap_keys_chunk(n, S->ds_host[krow].d, G, cnt_all, scratch);
             const size_t need_b = pdap_keys_bytes(n, G, chunk);
             if (need_b > S->keys_bytes) {
                 if (S->d_keys) S_TRY(cudaFreeAsync(S->d_keys, S->st));
