@@ -956,7 +956,9 @@ rrs_status rrs_depth_batched(rrs_ctx* ctx, const rrs_request* reqs, int32_t n_re
     P.tc_tune = &ctx->tc_tune;
     rrs_status s = build_plan(views, P);
     if (s != RRS_OK) return s;
-    const size_t bytes = plan_bytes(ctx, P);
+    size_keys(P, KEYS_SCRATCH_MIN);   // kept with the graph, once per graph
+    Carve sizing;
+    const size_t bytes = carve_plan(P, sizing);
     if (!budget_ok(ctx, bytes)) return fail(RRS_ERR_BUDGET, "batched workspace needs %zu bytes", bytes);
     rrs_ctx::GraphEntry G;
     G.key = key;
