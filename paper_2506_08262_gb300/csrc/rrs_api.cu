@@ -151,6 +151,7 @@ struct Plan {
     int rmax = 0;
     int max_ldx = 4, max_m = 0;
     int64_t hd_n = 0;   // largest n among the FP32 halfspace datasets
+    int hd_ldx = 4;     // and their largest row stride
     int64_t tot_ldx = 0, tot_d = 0, tot_u = 0, tot_m = 0;
     // tensor-core halfspace tasks, one group per K extent of the planes (64 or 128), each group one launch
     // per round whatever the datasets: every task's CTA takes its dataset's tensor map from maps
@@ -286,8 +287,9 @@ rrs_status build_plan(const std::vector<ReqView>& reqs, Plan& P)
         int G = 0;
         int cls = -1;
         const bool tc = R.kind == RRS_HALFSPACE && R.precision == RRS_PREC_SPLIT_BF16X3;
-        if (R.kind == RRS_HALFSPACE && !tc && D.ldx > 440)
-            return fail(RRS_ERR_UNSUPPORTED, "FP32 halfspace kernel stages 128 rows of d floats; d=%d too large", D.d);
+        if (R.kind == RRS_HALFSPACE && !tc && D.ldx > HD_MAX_LDX)
+            return fail(RRS_ERR_UNSUPPORTED, "FP32 halfspace kernel takes rows of at most %d floats; d=%d too large",
+                        HD_MAX_LDX, D.d);
         if (R.kind != RRS_HALFSPACE) {
             if (D.n > PDAP_MAX_N) return fail(RRS_ERR_UNSUPPORTED, "n too large for the selection kernel");
             int want = P.force_group;
@@ -351,6 +353,7 @@ rrs_status build_plan(const std::vector<ReqView>& reqs, Plan& P)
             // FP32 tasks: HD_ROWS consecutive (query, direction) rows of this request, across its queries
             const int64_t rows = R.nq * (int64_t)m;
             P.hd_n = std::max(P.hd_n, D.n);
+            P.hd_ldx = std::max(P.hd_ldx, D.ldx);
             for (int64_t g = 0; g < rows; g += HD_ROWS)
                 P.hd_tasks.push_back(
                     TaskDev{s_first + (int)(g / m), (int)(g % m), (int)std::min<int64_t>(HD_ROWS, rows - g), 0});
@@ -519,7 +522,7 @@ rrs_status enqueue_rounds(rrs_ctx* ctx, Plan& P, cudaStream_t st, bool capturing
         }
         if (P.n_hd[l] > 0) {
             StageTimer t(ctx, RRS_STAGE_HD_SIMT, st, capturing);
-            CUDA_TRY(launch_hd_simt(P.d_hd, P.n_hd[l], P.max_ldx, P.hd_n, P.d_slots, P.d_ds, P.U, P.yz, P.z64, P.res,
+            CUDA_TRY(launch_hd_simt(P.d_hd, P.n_hd[l], P.hd_ldx, P.hd_n, P.d_slots, P.d_ds, P.U, P.yz, P.z64, P.res,
                                     nullptr, ctx->d_err, st));
             ctx->stage_launches[RRS_STAGE_HD_SIMT]++;
             ctx->launches++;
@@ -1076,7 +1079,7 @@ rrs_status rrs_debug_round_depths(rrs_ctx* ctx, int64_t dataset_id, const void* 
                 CUDA_TRY(launch_hd_tc(P.tc[0].d, (int)P.tc[0].tasks.size(), P.tc[0].kp, P.tc[0].bn, 0, P.d_slots, P.d_ds, P.d_maps, P.U, P.yz,
                                       P.z64, P.res, band, ctx->d_err, st));
             else
-                CUDA_TRY(launch_hd_simt(P.d_hd, (int)P.hd_tasks.size(), P.max_ldx, 0, P.d_slots, P.d_ds, P.U, P.yz,
+                CUDA_TRY(launch_hd_simt(P.d_hd, (int)P.hd_tasks.size(), P.hd_ldx, 0, P.d_slots, P.d_ds, P.U, P.yz,
                                         P.z64, P.res, band, ctx->d_err, st));
         } else {
             for (size_t c = 0; c < P.pd_tasks.size(); ++c) {

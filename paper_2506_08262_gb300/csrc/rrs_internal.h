@@ -138,7 +138,10 @@ cudaError_t launch_gen(const TaskDev* tasks, int ntasks, const SlotDev* slots, c
 // consecutive slots they may run from one query into the next (j0 counts within the task's first query)
 // split_n: the largest n among the tasks' datasets, which lets a launch of few tasks split the points over more
 // CTAs (the result cells must then be zero, as launch_gen leaves them); 0: no split
+// max_ldx: the largest row stride among the tasks' datasets (sizes the shared memory), at most HD_MAX_LDX in a call;
+// wider rows are refused
 constexpr int HD_ROWS = 64;
+constexpr int HD_MAX_LDX = 440;
 constexpr int HD_PART_SHIFT = 48;   // bits of a count in a result cell shared by the parts of a split (n < 2^48)
 cudaError_t launch_hd_simt(const TaskDev* tasks, int ntasks, int max_ldx, int64_t split_n, const SlotDev* slots, const DsDev* ds,
                            const float* U, const double* yz, const double* z64, ResDev* res, int64_t* band_out,

@@ -196,7 +196,7 @@ extern "C" rrs_status rrs_depth_noalloc(const void* X, int64_t n, int32_t d, int
                             "n = %lld, n_queries = %lld and n_dirs = %d need more than the %zu bytes of the "
                             "static scratch of rrs_depth_noalloc",
                             (long long)n, (long long)n_queries, n_dirs, (size_t)RRS_NOALLOC_SCRATCH_BYTES);
-    if (kind == RRS_HALFSPACE && ldx > 440)
+    if (kind == RRS_HALFSPACE && ldx > HD_MAX_LDX)
         return noalloc_fail(RRS_ERR_UNSUPPORTED, "d=%d too large for the FP32 halfspace kernel", d);
     int G = 0, pd_variant = 0;
     size_t pd_smem = 0;

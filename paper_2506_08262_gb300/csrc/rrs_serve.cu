@@ -407,6 +407,7 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
         // tables of this step: gen tasks, halfspace tasks, selection tasks per launch key, argmin list
         std::vector<TaskDev> gen, hd;
         int64_t hd_n = 0;   // largest n among the FP32 halfspace datasets of the step
+        int hd_ldx = 4;     // and their largest row stride
         // (K extent of the planes, points per tile) -> tensor-core halfspace tasks
         std::map<std::pair<int, int>, std::vector<TaskDev>> tc;
         std::map<std::pair<int, int>, int64_t> tc_n;   // their largest n
@@ -447,6 +448,7 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
                     for (int j0 = 0; j0 < R->m; j0 += 128) v.push_back(TaskDev{slot, j0, std::min(128, R->m - j0), 0});
                 } else if (R->kind == RRS_HALFSPACE) {
                     hd_n = std::max(hd_n, D.n);
+                    hd_ldx = std::max(hd_ldx, D.ldx);
                     for (int j0 = 0; j0 < R->m; j0 += hper) hd.push_back(TaskDev{slot, j0, std::min(hper, R->m - j0), 0});
                 } else {
                     const int keys_row = sh.keys_gemm ? row : -1;
@@ -483,7 +485,7 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
         char* T = S->d_tab;
         S_TRY(launch_gen_slotround((const TaskDev*)(T + o_gen), (int)gen.size(), S->d_slots, S->d_p0, S->d_p1,
                                    S->d_z64, S->d_U, S->d_yz, S->d_res, S->max_ldx, S->st));
-        S_TRY(launch_hd_simt((const TaskDev*)(T + o_hd), (int)hd.size(), S->max_ldx, hd_n, S->d_slots, S->d_ds, S->d_U,
+        S_TRY(launch_hd_simt((const TaskDev*)(T + o_hd), (int)hd.size(), hd_ldx, hd_n, S->d_slots, S->d_ds, S->d_U,
                              S->d_yz, S->d_z64, S->d_res, nullptr, S->ctx->d_err, S->st));
         for (auto& to : o_tc)
             S_TRY(launch_hd_tc((const TaskDev*)(T + to.first), (int)tc[to.second].size(), to.second.first,
