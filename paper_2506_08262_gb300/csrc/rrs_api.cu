@@ -877,6 +877,7 @@ rrs_status rrs_depth(rrs_ctx* ctx, int64_t dataset_id, const void* Z, int64_t n_
         CUDA_TRY(cudaStreamSynchronize(st));
         if (!*ctx->h_flag) return RRS_OK;
         cudaMemsetAsync(ctx->d_err, 0, sizeof(int), st);
+        cudaStreamSynchronize(st);   // a call on another stream must not have its flag cleared by this
         return fail(RRS_ERR_INVALID_ARG, "Z holds a non-finite value or one of magnitude >= 2^64");
     };
     s = run_requests(ctx, reqs, st, 0, verdict);
@@ -1268,6 +1269,7 @@ rrs_status rrs_select_tc_tile(rrs_ctx* ctx, int64_t dataset_id, int32_t tile_poi
 rrs_status rrs_check(rrs_ctx* ctx, void* stream)
 {
     if (!ctx) return fail(RRS_ERR_INVALID_ARG, "NULL context");
+    std::lock_guard<std::mutex> lk(ctx->mu);   // h_flag is the context's
     CUDA_TRY(cudaSetDevice(ctx->device));
     return check_device_errors(ctx, (cudaStream_t)stream);
 }
