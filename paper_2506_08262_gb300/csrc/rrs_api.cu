@@ -772,6 +772,7 @@ static void drop_graphs(rrs_ctx* ctx)
     for (auto& g : ctx->graphs) {
         if (g.exec) cudaGraphExecDestroy(g.exec);
         cudaFree(g.ws);
+        ctx->used -= g.ws_bytes;
     }
     ctx->graphs.clear();
     cudaGetLastError();

@@ -33,3 +33,17 @@ def test_two_graphs_and_a_dataset_within_the_budget():
             if seed == 1:
                 assert torch.equal(depth, want)
         ctx.register(torch.randn(1_000_000, 40, device="cuda"))   # 176 MB more
+
+
+def test_dropped_graphs_give_their_bytes_back():
+    # every kernel choice drops the cached graphs; the budget holds three such workspaces at a time
+    rng = np.random.default_rng(3)
+    Z = torch.from_numpy(rng.standard_normal((100, 20), np.float32)).cuda()
+    depth = torch.empty(100, dtype=torch.float64, device="cuda")
+    stream = torch.cuda.current_stream()
+    with rrs.Context(0, 900_000_000) as ctx:
+        did = ctx.register(torch.from_numpy(rng.standard_normal((30_000, 20), np.float32)).cuda())
+        for i in range(6):
+            rrs.rrs_depth_batched(ctx.handle, [request(did, Z, depth, i)], True, stream)
+            rrs.rrs_check(ctx.handle, stream)
+            rrs.rrs_select_kernel(ctx.handle, did, 200, 2, 0)
