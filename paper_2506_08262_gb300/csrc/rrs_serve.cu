@@ -196,7 +196,10 @@ rrs_status step_table(rrs_server* S, size_t bytes)
 {
     if (bytes <= S->tab_bytes) return RRS_OK;
     if (S->d_tab) S_TRY(cudaFreeAsync(S->d_tab, S->st));
-    const size_t nb = std::max(bytes, S->tab_bytes * 2);
+    S->d_tab = nullptr;
+    const size_t old = S->tab_bytes;
+    S->tab_bytes = 0;   // should the allocation fail, the next step tries again
+    const size_t nb = std::max(bytes, old * 2);
     S_TRY(cudaMallocFromPoolAsync((void**)&S->d_tab, nb, S->ctx->pool, S->st));
     S->tab_bytes = nb;
     return RRS_OK;
@@ -509,6 +512,7 @@ rrs_status rrs_server_step(rrs_server* S, int32_t* active_queries_out, int32_t* 
             if (need_b > S->keys_bytes) {
                 if (S->d_keys) S_TRY(cudaFreeAsync(S->d_keys, S->st));
                 S->d_keys = nullptr;
+                S->keys_bytes = 0;
                 S_TRY(cudaMallocFromPoolAsync((void**)&S->d_keys, need_b, S->ctx->pool, S->st));
                 S->keys_bytes = need_b;
             }
