@@ -961,9 +961,16 @@ rrs_status rrs_depth_batched(rrs_ctx* ctx, const rrs_request* reqs, int32_t n_re
     P.tc_tune = &ctx->tc_tune;
     rrs_status s = build_plan(views, P);
     if (s != RRS_OK) return s;
-    size_keys(P, KEYS_SCRATCH_MIN);   // kept with the graph, once per graph
+    // the workspace is kept with the graph: large keys chunks for the first graphs of a context without a budget only
+    size_t kept = 0;
+    for (auto& g : ctx->graphs) kept += g.ws_bytes;
     Carve sizing;
-    const size_t bytes = carve_plan(P, sizing);
+    size_t bytes = carve_plan(P, sizing);
+    if (ctx->budget || kept + bytes > rrs_ctx::GRAPH_KEEP) {
+        size_keys(P, KEYS_SCRATCH_MIN);
+        Carve again;
+        bytes = carve_plan(P, again);
+    }
     if (!budget_ok(ctx, bytes)) return fail(RRS_ERR_BUDGET, "batched workspace needs %zu bytes", bytes);
     rrs_ctx::GraphEntry G;
     G.key = key;

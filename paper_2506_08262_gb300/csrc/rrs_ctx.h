@@ -45,6 +45,8 @@ struct rrs_ctx {
     // call), up to POOL_KEEP bytes; a context with a budget keeps nothing.  Given back by rrs_destroy.
     static constexpr uint64_t POOL_KEEP = (uint64_t)2 << 30;
     cudaMemPool_t pool = nullptr;
+    // workspace bytes of cached graphs up to which a further one takes large keys chunks
+    static constexpr uint64_t GRAPH_KEEP = (uint64_t)2 << 30;
     int* h_flag = nullptr;   // pinned: device-side flags read back without a staged copy
     std::mutex mu;
     // cached captured graphs of batched calls (keyed by the request bytes)

@@ -165,8 +165,9 @@ cudaError_t launch_pdap(const TaskDev* tasks, int ntasks, size_t smem, int group
 size_t pdap_keys_bytes(int n, int group, int ntasks);
 // Bytes of selection keys formed at a time (one chunk of tasks: a keys launch, then the selection on them).  A chunk's
 // launches end in waves that are partly empty, so chunks are large: n = 100,000 at d = 100 took 117 / 89 / 74 / 66 ms
-// with 64 / 128 / 256 / 512 MB.  Where the context's budget has no room for KEYS_SCRATCH_BYTES, and in a workspace that
-// a captured graph keeps, the plan takes KEYS_SCRATCH_MIN.
+// with 64 / 128 / 256 / 512 MB.  Where the context's budget has no room for KEYS_SCRATCH_BYTES the plan takes
+// KEYS_SCRATCH_MIN; so does a captured graph, which keeps its workspace, under a budget or where the context's graphs
+// hold rrs_ctx::GRAPH_KEEP (32 datasets of up to 50,000 points: 38.3 ms a call with large chunks, 39.1 with small ones).
 constexpr size_t KEYS_SCRATCH_BYTES = (size_t)1 << 30, KEYS_SCRATCH_MIN = (size_t)256 << 20;
 // Tasks of one keys launch: at most `bytes` of keys and what its grid holds, one at least.
 int pdap_keys_chunk(int n, int d, int group, int64_t ntasks, size_t bytes);
