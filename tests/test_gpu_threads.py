@@ -23,7 +23,7 @@ def calls(d, n, kind, nq, reps, start, out):
             start.wait(60)
             seen = set()
             for _ in range(reps):
-                depth, _, best = ctx.depth(did, Z, kind, 40, 5, 0.7, 3)
+                depth, _, best = ctx.depth(did, Z, kind, 200, 100, 0.7, 3)
                 seen.add((depth.cpu().numpy().tobytes(), best.cpu().numpy().tobytes()))
             out.append(len(seen))
     except rrs.RRSError as e:
@@ -32,9 +32,10 @@ def calls(d, n, kind, nq, reps, start, out):
 
 @pytest.mark.parametrize("kind", [rrs.RRS_HALFSPACE, rrs.RRS_PROJECTION])
 def test_wide_and_narrow_datasets_side_by_side(kind):
-    # shared memory of a launch grows with d (directions staged) and with n (selection keys and buckets)
+    # shared memory of a launch grows with d (directions staged) and with n (selection keys and buckets); 100 rounds a
+    # call keep both threads launching
     start, out = threading.Barrier(2), []
-    args = [(400, 300, kind, 4, 300, start, out), (2, 9000, kind, 4, 300, start, out)]
+    args = [(400, 300, kind, 4, 60, start, out), (2, 9000, kind, 4, 60, start, out)]
     threads = [threading.Thread(target=calls, args=a) for a in args]
     for t in threads:
         t.start()
