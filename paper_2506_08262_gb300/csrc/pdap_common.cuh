@@ -270,15 +270,17 @@ __device__ void gpick(const Grp<GS>& q, const float* buf, const int* ib, int cnt
 // plus its rank within its own bucket.
 constexpr int NB2 = 256;
 static_assert(NB2 + 2 * CAP1H == NB, "D_P runs in the histogram area: NB2 counters, then CAP1H values and CAP1H indices");
-template <int GS, class CT, int TCAP = CAP>
-__device__ void gpick_wide(const Grp<GS>& q, const float* buf, const int* ib, int cnt, int s1, int s2, float lo,
+// False, and nothing picked, where the values have no range or the ranks' buckets hold more pairs than (tb, ti).
+template <int GS, class CT, int TCAP>
+__device__ bool gpick_bins(const Grp<GS>& q, const float* buf, const int* ib, int cnt, int s1, int s2, float lo,
                            float hi, unsigned* h2, float* tb, int* ti, CT& C, float& o1, float& o2, int& i1,
                            int& i2)
 {
-    if (cnt <= 64 || !(lo < hi)) {
+    if (cnt <= 64) {
         gpick(q, buf, ib, cnt, s1, s2, C, o1, o2, i1, i2);
-        return;
+        return true;
     }
+    if (!(lo < hi)) return false;
     float scale = __fdiv_rn((float)NB2, __fsub_rn(hi, lo));
     if (!(scale <= FLT_MAX)) scale = FLT_MAX;
     for (int b = q.t; b < NB2; b += GS) h2[b] = 0u;
@@ -326,10 +328,7 @@ __device__ void gpick_wide(const Grp<GS>& q, const float* buf, const int* ib, in
     q.sync();
     const int b1 = C.f_b1[q.g], c1 = C.f_c1[q.g], b2 = C.f_b2[q.g];
     const int n2 = C.f_c2[q.g] + (int)h2[b2] - c1;
-    if (n2 > TCAP) {   // the rank buckets hold more pairs than (tb, ti): rank the whole set
-        gpick(q, buf, ib, cnt, s1, s2, C, o1, o2, i1, i2);
-        return;
-    }
+    if (n2 > TCAP) return false;
     for (int t = q.t; t < cnt; t += GS) {
         const float v = buf[t];
         const int b = bk(v);
@@ -343,6 +342,17 @@ __device__ void gpick_wide(const Grp<GS>& q, const float* buf, const int* ib, in
     }
     q.sync();
     gpick(q, tb, ti, n2, s1 - c1, s2 - c1, C, o1, o2, i1, i2);
+    return true;
+}
+
+// The same for every set: the whole of it is ranked where gpick_bins picks nothing.
+template <int GS, class CT, int TCAP = CAP>
+__device__ __forceinline__ void gpick_wide(const Grp<GS>& q, const float* buf, const int* ib, int cnt, int s1, int s2,
+                                           float lo, float hi, unsigned* h2, float* tb, int* ti, CT& C, float& o1,
+                                           float& o2, int& i1, int& i2)
+{
+    if (!gpick_bins<GS, CT, TCAP>(q, buf, ib, cnt, s1, s2, lo, hi, h2, tb, ti, C, o1, o2, i1, i2))
+        gpick(q, buf, ib, cnt, s1, s2, C, o1, o2, i1, i2);
 }
 
 // Generic exact selection of rank q1 over one direction's values f(0..L-1),
