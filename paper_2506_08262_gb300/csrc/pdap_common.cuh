@@ -358,15 +358,13 @@ __device__ __forceinline__ void gpick_wide(const Grp<GS>& q, const float* buf, c
 // Generic exact selection of rank q1 over one direction's values f(0..L-1),
 // all in [lo, hi], by iterated bucketing (the fallback path); hist, buf and ibuf are the
 // direction's own areas.  Returns the value and its point index.  One rank at a time: its bucket narrows every
-// round, where the run of two ranks in two groups of equal values would never shrink.
+// round, where the run of two ranks in two groups of equal values would never shrink.  Rank q2 >= q1 comes along
+// where it lies in the group that ends the search (returns true).
 template <int GS, class CT, class F, int FBN = FB_NB, int FBC = FB_CAP>
-__device__ __noinline__ void gselect1(const Grp<GS>& q, F f, int L, int q1, float lo, float hi, unsigned* hist, float* buf, int* ibuf,
-                         CT& C, float& v1, int& i1, int* err)
+__device__ __noinline__ bool gselect1(const Grp<GS>& q, F f, int L, int q1, int q2, float lo, float hi, unsigned* hist, float* buf,
+                         int* ibuf, CT& C, float& v1, int& i1, float& v2, int& i2, int* err)
 {
-    const int q2 = q1;
-    float v2;
-    int i2;
-    int below = 0;
+    int below = 0, left = L;   // values below the candidates, and candidates
     for (int iter = 0; iter < 24; ++iter) {
         if (!(lo < hi)) {
             // every remaining candidate equals lo: the rank holds that value, taken at the smallest point index
@@ -382,8 +380,10 @@ __device__ __noinline__ void gselect1(const Grp<GS>& q, F f, int L, int q1, floa
             q.sync();
             v1 = lo;
             i1 = C.gi[q.g] == 0x7FFFFFFF ? -1 : C.gi[q.g];
+            v2 = v1;
+            i2 = i1;
             q.sync();
-            return;
+            return q2 - below < left;
         }
         float scale = __fdiv_rn((float)FBN, __fsub_rn(hi, lo));
         if (!(scale <= FLT_MAX)) scale = FLT_MAX;
@@ -395,16 +395,15 @@ __device__ __noinline__ void gselect1(const Grp<GS>& q, F f, int L, int q1, floa
         }
         q.sync();
         int b1, c1, b2, c2;
-        gfind<GS, CT, FBN>(q, hist, q1 - below, q2 - below, C, b1, c1, b2, c2);
-        const int cnt = c2 + (int)hist[b2] - c1;
+        gfind<GS, CT, FBN>(q, hist, q1 - below, q1 - below, C, b1, c1, b2, c2);
+        const int cnt = (int)hist[b1];
         if (q.t == 0) C.gn[q.g] = 0;
         q.sync();
         if (cnt <= FBC) {
             for (int i = q.t; i < L; i += GS) {
                 const float a = f(i);
                 if (a >= lo && a <= hi) {
-                    const int b = bucket<FBN>(a, lo, scale);
-                    if (b >= b1 && b <= b2) {
+                    if (bucket<FBN>(a, lo, scale) == b1) {
                         const int pos = atomicAdd(&C.gn[q.g], 1);
                         if (pos < FBC) {
                             buf[pos] = a;
@@ -414,15 +413,15 @@ __device__ __noinline__ void gselect1(const Grp<GS>& q, F f, int L, int q1, floa
                 }
             }
             q.sync();
-            gpick(q, buf, ibuf, cnt, q1 - below - c1, q2 - below - c1, C, v1, v2, i1, i2);
-            return;
+            const int r1 = q1 - below - c1, r2 = q2 - below - c1;
+            gpick(q, buf, ibuf, cnt, r1, r2 < cnt ? r2 : r1, C, v1, v2, i1, i2);
+            return r2 < cnt;
         }
         float nlo = FLT_MAX, nhi = -FLT_MAX;
         for (int i = q.t; i < L; i += GS) {
             const float a = f(i);
             if (a >= lo && a <= hi) {
-                const int b = bucket<FBN>(a, lo, scale);
-                if (b >= b1 && b <= b2) {
+                if (bucket<FBN>(a, lo, scale) == b1) {
                     nlo = fminf(nlo, a);
                     nhi = fmaxf(nhi, a);
                 }
@@ -430,10 +429,12 @@ __device__ __noinline__ void gselect1(const Grp<GS>& q, F f, int L, int q1, floa
         }
         gminmax(q, nlo, nhi, C, lo, hi);
         below += c1;
+        left = cnt;
     }
     if (q.t == 0) atomicOr(err, ERR_SELECT_ITER);
-    v1 = __int_as_float(0x7FC00000);
-    i1 = -1;
+    v1 = v2 = __int_as_float(0x7FC00000);
+    i1 = i2 = -1;
+    return true;
 }
 
 // Two ranks q1 <= q2 by gselect1.
@@ -441,10 +442,10 @@ template <int GS, class CT, class F>
 __device__ __forceinline__ void gselect(const Grp<GS>& q, F f, int L, int q1, int q2, float lo, float hi, unsigned* hist,
                                         float* buf, int* ibuf, CT& C, float& v1, float& v2, int& i1, int& i2, int* err)
 {
-    gselect1(q, f, L, q1, lo, hi, hist, buf, ibuf, C, v1, i1, err);
-    v2 = v1;
-    i2 = i1;
-    if (q2 != q1) gselect1(q, f, L, q2, lo, hi, hist, buf, ibuf, C, v2, i2, err);
+    if (gselect1(q, f, L, q1, q2, lo, hi, hist, buf, ibuf, C, v1, i1, v2, i2, err)) return;
+    float w;
+    int j;
+    gselect1(q, f, L, q2, q2, lo, hi, hist, buf, ibuf, C, v2, i2, w, j, err);
 }
 
 // One direction's keys held in an array: shared memory (resident keys) or device memory (keys formed
