@@ -159,11 +159,11 @@ __device__ __forceinline__ float key_halves(const float* u, const float* x)
 }
 
 // Pass A of k_pdap2 for d <= 16 (D4 = d rounded up to 4, the directions uu in registers): the keys of G
-// directions for the points t0, t0 + 1, then step further on, stored (unless STREAM) and counted in the
+// directions for the points t0, t0 + 1, then step further on, stored and counted in the
 // directions' histograms.  Two points per thread: from the dataset's columns Xt (dim l of point i at
 // l * colst + i) their coordinates come as one 8-byte load per dim, side by side over the lanes; without columns
 // from the padded rows.
-template <int G, int D4, bool STREAM>
+template <int G, int D4>
 __device__ __forceinline__ void pass_a_pairs(const DsDev& D, int t0, int step, int n, int kst, const float (&uu)[G][D4],
                                              const float (&sc)[G], const float (&of)[G], float* keys, unsigned* hist)
 {
@@ -198,17 +198,16 @@ __device__ __forceinline__ void pass_a_pairs(const DsDev& D, int t0, int step, i
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             const float ka = key_halves<D4>(uu[g], xa), kb = key_halves<D4>(uu[g], xb);
-            if (!STREAM) *reinterpret_cast<float2*>(keys + (size_t)g * kst + i) = make_float2(ka, kb);   // kst is even
+            *reinterpret_cast<float2*>(keys + (size_t)g * kst + i) = make_float2(ka, kb);   // kst is even
             atomicAdd(&hist[g * NB + bucket_m(ka, sc[g], of[g])], 1u);
             if (two) atomicAdd(&hist[g * NB + bucket_m(kb, sc[g], of[g])], 1u);
         }
     }
 }
 
-// One direction's keys recomputed from the FP32 rows of X with the projection pass's arithmetic
-// (two half chains for d <= 16, one sequential FMA chain otherwise), so every pass sees the values
-// a resident key would hold.  u: the direction in shared memory, dp4 floats (zero padded).
-template <int DP4>
+// One direction's keys recomputed from the FP32 rows of X with the projection pass's arithmetic (d > 16: one sequential
+// FMA chain), so every pass sees the values a resident key would hold.  u: the direction in shared memory, dp4 floats
+// (zero padded).
 struct KeysRecomputed {
     const float* X;
     const float* u;
@@ -216,24 +215,6 @@ struct KeysRecomputed {
     __device__ __forceinline__ float get(int i) const
     {
         const float4* xr = reinterpret_cast<const float4*>(X + (int64_t)i * ldx);
-        if (DP4 > 0) {
-            constexpr int D4 = DP4 > 0 ? DP4 : 4;
-            float xv[D4], uv[D4];
-#pragma unroll
-            for (int c = 0; c < D4 / 4; ++c) {
-                const float4 t4 = xr[c];
-                const float4 u4 = *reinterpret_cast<const float4*>(u + 4 * c);
-                xv[4 * c] = t4.x;
-                xv[4 * c + 1] = t4.y;
-                xv[4 * c + 2] = t4.z;
-                xv[4 * c + 3] = t4.w;
-                uv[4 * c] = u4.x;
-                uv[4 * c + 1] = u4.y;
-                uv[4 * c + 2] = u4.z;
-                uv[4 * c + 3] = u4.w;
-            }
-            return key_halves<D4>(uv, xv);
-        }
         float acc = 0.f;
         for (int l = 0; l < dp4; l += 4) {
             const float4 x = xr[l >> 2];
@@ -608,12 +589,11 @@ __device__ __forceinline__ void select_dir(const Grp<GS>& q, const K& y, Ctl& C,
 }
 
 // Every live direction of the CTA: group g of cta_threads<G>() / G threads handles direction g alone,
-// on its keys in shared memory or (STREAM) on keys formed by launch_pdap_keys in global memory (kin), else
-// on keys recomputed from X.
-template <int G, int DP4, bool STREAM>
+// on its keys in shared memory or (STREAM) recomputed from X.
+template <int G, bool STREAM>
 __device__ __forceinline__ void select_dirs(Ctl& C, const float* keys, const float* uS, unsigned* hist, float* buf,
-                                            int* ibuf, int n, int npad, int kst, bool ap, const DsDev& D, int GA,
-                                            int64_t roff, ResDev* __restrict__ res, int* err, const float* kin)
+                                            int* ibuf, int n, int kst, bool ap, const DsDev& D, int GA,
+                                            int64_t roff, ResDev* __restrict__ res, int* err)
 {
     constexpr int GS = cta_threads<G>() / G;   // threads per direction group
     const int tid = threadIdx.x;
@@ -624,11 +604,8 @@ __device__ __forceinline__ void select_dirs(Ctl& C, const float* keys, const flo
     float* B0 = buf + (size_t)g * (CAP + CAP1);   // two gather runs, contiguous (FB_CAP for the fallback)
     int* I0 = ibuf + (size_t)g * (CAP + CAP1);    // the point index of every gathered key
     const float* u = uS + (size_t)g * D.ldx;
-    if (STREAM && kin) {
-        const KeysArray y{kin + ((size_t)blockIdx.x * G + g) * npad};
-        select_dir<GS>(q, y, C, H, B0, I0, n, ap, D, roff, res, err);
-    } else if (STREAM) {
-        const KeysRecomputed<DP4> y{D.X32, u, D.ldx, DP4 ? DP4 : ((D.d + 3) & ~3)};
+    if (STREAM) {
+        const KeysRecomputed y{D.X32, u, D.ldx, (D.d + 3) & ~3};
         select_dir<GS>(q, y, C, H, B0, I0, n, ap, D, roff, res, err);
     } else {
         const KeysArray y{keys + (size_t)g * kst};
@@ -638,9 +615,9 @@ __device__ __forceinline__ void select_dirs(Ctl& C, const float* keys, const flo
 
 // G: directions per CTA (compile time); DP4: d rounded up to 4 when <= 16 (the
 // directions are then held in registers), 0 for any d; STREAM: no keys in shared
-// memory, every pass reads them from kin or recomputes them from X.
+// memory, every pass recomputes them from X (d > 16 only).
 // kin: optional precomputed keys, G x npad per task in launch order (launch_pdap_keys), read instead of
-// projecting
+// projecting (not with STREAM)
 template <int G, int DP4, bool STREAM>
 __global__ void __launch_bounds__(cta_threads<G>(), (G >= 4 ? 1 : 2)) k_pdap2(const TaskDev* __restrict__ tasks, const SlotDev* __restrict__ slots,
                                                  const DsDev* __restrict__ dsets, const float* __restrict__ U,
@@ -742,8 +719,8 @@ __global__ void __launch_bounds__(cta_threads<G>(), (G >= 4 ? 1 : 2)) k_pdap2(co
                 atomicAdd(&hist[g * NB + bucket_m(acc[g], sc[g], of[g])], 1u);
             }
         };
-        if (kin) {
-            // keys formed by k_keys (same arithmetic as the projection below): count (and copy unless STREAM)
+        if (!STREAM && kin) {
+            // keys formed by k_keys (same arithmetic as the projection below): count and copy
             const float4* src = reinterpret_cast<const float4*>(kin + (size_t)blockIdx.x * G * npad);
             for (int e = tid; e < G * npad / 4; e += NTK) {
                 const int g = e / (npad / 4), i = 4 * (e - g * (npad / 4));
@@ -753,7 +730,7 @@ __global__ void __launch_bounds__(cta_threads<G>(), (G >= 4 ? 1 : 2)) k_pdap2(co
 #pragma unroll
                 for (int h = 0; h < 4; ++h) {
                     if (i + h < n) {
-                        if (!STREAM) keys[(size_t)g * kst + i + h] = kv[h];
+                        keys[(size_t)g * kst + i + h] = kv[h];
                         atomicAdd(&hist[g * NB + bucket_m(kv[h], sc[g], of[g])], 1u);
                     }
                 }
@@ -776,7 +753,7 @@ __global__ void __launch_bounds__(cta_threads<G>(), (G >= 4 ? 1 : 2)) k_pdap2(co
                 u2[1][l] = ub[l];
             }
             const float s2[2] = {sc[2 * pair], sc[2 * pair + 1]}, o2[2] = {of[2 * pair], of[2 * pair + 1]};
-            pass_a_pairs<2, D4, STREAM>(D, 2 * (tid >> 1), NTK, n, kst, u2, s2, o2, keys + (size_t)(2 * pair) * kst,
+            pass_a_pairs<2, D4>(D, 2 * (tid >> 1), NTK, n, kst, u2, s2, o2, keys + (size_t)(2 * pair) * kst,
                                         hist + 2 * pair * NB);
         } else if (DP4 > 0) {
             constexpr int D4 = DP4 > 0 ? DP4 : 4;
@@ -791,7 +768,7 @@ __global__ void __launch_bounds__(cta_threads<G>(), (G >= 4 ? 1 : 2)) k_pdap2(co
                     uu[g][4 * c + 2] = u4.z;
                     uu[g][4 * c + 3] = u4.w;
                 }
-            pass_a_pairs<G, D4, STREAM>(D, 2 * tid, 2 * NTK, n, kst, uu, sc, of, keys, hist);
+            pass_a_pairs<G, D4>(D, 2 * tid, 2 * NTK, n, kst, uu, sc, of, keys, hist);
         } else {
             for (int i = tid; i < n; i += NTK) {
                 const float4* xr = reinterpret_cast<const float4*>(D.X32 + (int64_t)i * ldx);
@@ -815,7 +792,7 @@ __global__ void __launch_bounds__(cta_threads<G>(), (G >= 4 ? 1 : 2)) k_pdap2(co
     }
     __syncthreads();
 
-    select_dirs<G, DP4, STREAM>(C, keys, uS, hist, buf, ibuf, n, npad, kst, ap, D, GA, S.roff + T.j0, res, err, kin);
+    select_dirs<G, STREAM>(C, keys, uS, hist, buf, ibuf, n, kst, ap, D, GA, S.roff + T.j0, res, err);
 }
 
 }  // namespace
@@ -833,32 +810,15 @@ size_t pdap_smem_limit()
     return 232448 - sizeof(Ctl) - 64 - 256;
 }
 
-size_t pdap_two_per_sm_limit()
+// Directions per CTA of the allocation-free call for d > 16: the most of 1, 2, 4 whose keys fit, 0 if none do.  The
+// projection pass re-reads X (4 d bytes per point) for every G directions (measured at n = 10,000: d = 50 1.27x,
+// d = 150 1.68x faster with G = 4 than G = 2).
+int pdap_max_group(int n, int ldx, int m)
 {
-    // 228 KB per SM shared by two CTAs, each also holding 1 KB of reserved and ~1 KB of static memory
-    return 112 * 1024;
-}
-
-int pdap_max_group(int n, int ldx, int m, int d, bool keys_in, bool allow_stream)
-{
-    // G in {1, 2, 4}: the largest G that fits two CTAs per SM when that is at least 2.  Below that the
-    // keys go outside shared memory (0: formed once per round by a keys kernel, read at every pass),
-    // which keeps four directions per SM in flight instead of one or two (measured on the 256-dataset
-    // batched workload: the selection stage 8.2 s -> 5.4 s, identical results); callers that cannot
-    // hold the keys elsewhere (allow_stream false) take the largest G that fits one CTA per SM.
-    // Exception: for d > 16 with keys formed inside the kernel the projection pass re-reads X (4 d
-    // bytes per point) for every G directions, so there the largest G that fits wins (measured at
-    // n = 10,000: d = 50 1.27x, d = 150 1.68x faster with G = 4 than G = 2).
-    const size_t one = pdap_smem_limit(), two = pdap_two_per_sm_limit();
-    int g_one = 0, g_two = 0;
-    for (int g = 1; g <= MAXG && g <= m; g *= 2) {
-        const size_t need = pdap_smem_bytes(n, g, ldx);
-        if (need <= one) g_one = g;
-        if (need <= two) g_two = g;
-    }
-    if (pdap_dp4_class(d) == 0 && !keys_in) return g_one;
-    if (g_two >= 2 || (g_two >= 1 && m < 2)) return g_two;
-    return allow_stream ? 0 : g_one;
+    int most = 0;
+    for (int g = 1; g <= MAXG && g <= m; g *= 2)
+        if (pdap_smem_bytes(n, g, ldx) <= pdap_smem_limit()) most = g;
+    return most;
 }
 
 // Keys of a block of tasks (G directions each, all of one dataset) for every point, as a tiled FP32
@@ -1030,17 +990,17 @@ static cudaError_t launch_t(const TaskDev* tasks, int ntasks, size_t smem, const
     return cudaGetLastError();
 }
 
-template <int G, bool STREAM>
+template <int G>
 static cudaError_t launch_g(int dp4, const TaskDev* tasks, int ntasks, size_t smem, const SlotDev* slots,
                             const DsDev* ds, const float* U, const double* yz, ResDev* res, int* err, const float* kin,
                             cudaStream_t st)
 {
     switch (dp4) {
-    case 4: return launch_t<G, 4, STREAM>(tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
-    case 8: return launch_t<G, 8, STREAM>(tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
-    case 12: return launch_t<G, 12, STREAM>(tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
-    case 16: return launch_t<G, 16, STREAM>(tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
-    default: return launch_t<G, 0, STREAM>(tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
+    case 4: return launch_t<G, 4, false>(tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
+    case 8: return launch_t<G, 8, false>(tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
+    case 12: return launch_t<G, 12, false>(tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
+    case 16: return launch_t<G, 16, false>(tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
+    default: return launch_t<G, 0, false>(tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
     }
 }
 
@@ -1079,9 +1039,9 @@ static cudaError_t launch_select(const TaskDev* tasks, int ntasks, size_t smem, 
         return launch_t<PDAP_STREAM_GROUP, 0, true>(tasks, ntasks, smem, slots, ds, U, yz, res, err, nullptr, st);
     }
     switch (group) {
-    case 1: return launch_g<1, false>(dp4, tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
-    case 2: return launch_g<2, false>(dp4, tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
-    case 4: return launch_g<4, false>(dp4, tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
+    case 1: return launch_g<1>(dp4, tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
+    case 2: return launch_g<2>(dp4, tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
+    case 4: return launch_g<4>(dp4, tasks, ntasks, smem, slots, ds, U, yz, res, err, kin, st);
     default: return cudaErrorInvalidValue;
     }
 }

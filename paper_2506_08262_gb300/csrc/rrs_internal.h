@@ -88,7 +88,7 @@ enum : int {
 // Near-tie band factors: a point is re-checked exactly when
 // |t| <= gamma * (|x| + |z|), t the fast projection difference.
 // FP32 path: |fl32 dot - exact| <= gamma_d sum|u x| (gamma_d ~ d 2^-24), plus one rounding of x to FP32
-// (FP64 inputs), of y_z to FP32 and of the final difference; twice that sum for slack.
+// (FP64 inputs) and of y_z, from which the chain starts, to FP32; twice that sum for slack.
 __host__ __device__ inline float band_gamma_fp32(int d) { return (float)((double)(d + 4) * 0x1p-23); }
 float band_gamma_tc(int kp);
 // cuTensorMapEncodeTiled, looked up once through the runtime (NULL when unavailable)
@@ -161,7 +161,7 @@ cudaError_t launch_pdap(const TaskDev* tasks, int ntasks, size_t smem, int group
 // Keys of ntasks selection tasks (all of one dataset) into keys (pdap_keys_bytes), for
 // launch_pdap(..., kin = keys) on the same task range, with the selection kernel's own key arithmetic:
 // a tiled FP32 GEMM for d > 16 (where forming the keys inside the selection kernel re-reads X for every
-// G directions), two half chains per key for d <= 16 (used when the keys do not fit shared memory)
+// G directions), two half chains per key for d <= 16 (where keys in device memory are asked for)
 size_t pdap_keys_bytes(int n, int group, int ntasks);
 // Bytes of selection keys formed at a time (one chunk of tasks: a keys launch, then the selection on them).  A chunk's
 // launches end in waves that are partly empty, so chunks are large: n = 100,000 at d = 100 took 117 / 89 / 74 / 66 ms
@@ -205,8 +205,8 @@ cudaError_t launch_moments(const float* X32, int64_t n, int d, int ldx, float* c
 cudaError_t launch_check_finite(const void* Z, int dtype, int64_t count, int* bad, cudaStream_t st);
 size_t pdap_smem_bytes(int n, int group, int ldx, bool stream = false);
 size_t pdap_smem_limit();
-// preferred resident G; 0: keys outside shared memory (when allow_stream, or when none fits)
-int pdap_max_group(int n, int ldx, int m, int d, bool keys_in = false, bool allow_stream = false);
+// directions per CTA of the allocation-free call for d > 16, 0 where none fits with its keys
+int pdap_max_group(int n, int ldx, int m);
 
 // Selection-kernel variant bit: no keys in shared memory, every pass recomputes them from X (the allocation-free
 // entry point with d > 16 where they do not fit).  Such launches take PDAP_STREAM_GROUP directions per CTA.

@@ -210,7 +210,7 @@ extern "C" rrs_status rrs_depth_noalloc(const void* X, int64_t n, int32_t d, int
             G = (m + ctas - 1) / ctas;   // a query's directions spread evenly over its CTAs
             pd_variant = sh.variant;
             pd_smem = sh.smem;
-        } else if (int Gr = pdap_max_group((int)n, ldx, m, d)) {
+        } else if (int Gr = pdap_max_group((int)n, ldx, m)) {
             G = Gr;
             pd_variant = pdap_dp4_class(d);
             pd_smem = pdap_smem_bytes((int)n, G, ldx);
