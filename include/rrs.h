@@ -111,9 +111,11 @@ rrs_status rrs_free(rrs_ctx* ctx, int64_t dataset_id);
  *   and of z.  For d <= 16 the keys are re-formed from the data at both passes
  *   of the selection; for larger d they are formed once per round in device
  *   memory (up to 1 GB of scratch, 256 MB where the context's budget has no room
- *   for more, taken in chunks) and read back at both passes.  The arithmetic is
- *   the same in every form, so results do not depend on which ran.  n is limited
- *   to 2^31 - 64 for projection depths.
+ *   for more, taken in chunks) and read back at both passes.  Where many keys are
+ *   alike (repeated points, a dense core) and for n above about 1.9 million a
+ *   direction takes further passes.  The arithmetic is the same in every form, so
+ *   results do not depend on which ran.  n is limited to 2^31 - 64 for projection
+ *   depths.
  * Outputs (each n_queries long, or n_queries*r for round_choice_out):
  *   depth_out[q]   final depth D_min (double).                      required
  *   count_out[q]   halfspace: min(#<=, #>=) at D_min, else -1.        optional
@@ -164,13 +166,16 @@ typedef struct rrs_request {
  * (Sec. 4: directions are independent within a round, queries are
  * independent).  Results are identical to calling rrs_depth on each request
  * alone with the request's precision.  Halfspace requests with
- * RRS_PREC_SPLIT_BF16X3 run on the tensor cores, one launch per dataset and
- * round covering all of that dataset's such requests; their counts equal the
+ * RRS_PREC_SPLIT_BF16X3 run on the tensor cores, one launch per round and K
+ * extent of the planes covering all such requests; their counts equal the
  * FP32 path's (both are exact).  Requests may have different r; a request
  * leaves the batch when its rounds are done.
  *   reqs: host array of n_requests descriptors; all pointers inside are
  *   device pointers.  use_graph != 0 captures the launch sequence into a
- *   CUDA graph that is replayed on later calls with identical descriptors.
+ *   CUDA graph that is replayed on later calls with identical descriptors; the
+ *   context keeps the graph and its workspace until it is destroyed or a kernel
+ *   choice changes (selection keys in it: 256 MB at a time, up to 1 GB while the
+ *   context has no budget and its graphs hold less than 2 GB in all).
  * Errors: as rrs_depth.  Stream-ordered on `stream`.
  */
 rrs_status rrs_depth_batched(rrs_ctx* ctx, const rrs_request* reqs, int32_t n_requests,
@@ -287,12 +292,14 @@ uint64_t rrs_launch_count(rrs_ctx* ctx);
 
 /* Pipeline stages timed by the profiler (one slot each in rrs_profile_read). */
 #define RRS_STAGE_PREP 0      /* query conversion and state initialisation */
-#define RRS_STAGE_GEN 1       /* direction generation (Alg. S1 / S4) and y_z */
+#define RRS_STAGE_GEN 1       /* direction generation (Alg. S1 / S4) and y_z: round 1, and the later rounds of calls
+                                 with more than 128 directions per round */
 #define RRS_STAGE_HD_SIMT 2   /* halfspace counts, FP32 CUDA-core projection */
 #define RRS_STAGE_HD_TC 3     /* halfspace counts, tcgen05 split-BF16x3 projection */
 #define RRS_STAGE_PDAP 4      /* projection / asymmetric projection depth (selection) */
-#define RRS_STAGE_ARGMIN 5    /* round minimum and pole update (Alg. 1 steps 4-6) */
-#define RRS_STAGE_KEYS 6      /* selection keys formed once per round (d > 16, or n beyond shared memory) */
+#define RRS_STAGE_ARGMIN 5    /* round minimum and pole update (Alg. 1 steps 4-6), with the next round's directions
+                                 and y_z in the same launch where a round has at most 128 */
+#define RRS_STAGE_KEYS 6      /* selection keys formed once per round (d > 16, or RRS_SELECT_STREAM asked for) */
 #define RRS_NSTAGES 7
 
 /*
