@@ -1009,9 +1009,9 @@ __device__ __forceinline__ void rf_red(unsigned hb, int raw, bool take)
 }
 
 // One direction's keys k of the points i, i + 1 (then i + 2, i + 3; the next four 128 further on) in the current pass, by
-// a whole warp.  Bound by its instructions, some 35 a key with forming it, where the first passes take 23 together
-// (RF_PIVOT: about 12).  Where many keys are alike most candidates share a sub-bucket: those in the one of the warp's
-// first count with one reduction.
+// a whole warp.  Bound by its instructions: a pass takes about as long as the first two together (10,000 points in 10
+// dims, 50,000 directions: 1.0 ms against 1.1), RF_PIVOT less than half.  Where many keys are alike most candidates
+// share a sub-bucket: those in the one of the warp's first count with one reduction.
 template <int S>
 __device__ __forceinline__ void rf_keys(SelRef& F, const SelPar& par, unsigned* H, int nb, const unsigned long long (&k)[S],
                                         unsigned i, unsigned n)
@@ -1248,7 +1248,8 @@ __device__ __noinline__ void sel_refine_k(const TaskDev* tasks, int G, const Slo
 
 // Keys in device memory (kin: G x npad per task in launch order, formed by launch_pdap_keys): one block of GS
 // threads per direction, so directions never wait for one another and a block's few barriers are its own.
-// Bound by the shared-memory reductions and the issue slots of the two passes, about 14 instructions per key.
+// Measured at n = 10,000 (26,840 directions, 449 us): 30 instructions a key, the shared-memory pipe at 66% of its
+// wavefronts (half of them the reductions), issue slots at 48%; warps wait for keys from memory first.
 template <int GS>
 __global__ void __launch_bounds__(GS, 1024 / GS) k_select(const TaskDev* __restrict__ tasks, int G,
                                                const SlotDev* __restrict__ slots, const DsDev* __restrict__ dsets,
@@ -1497,7 +1498,9 @@ __device__ __noinline__ void sel_refine_x(const TaskDev* tasks, const SlotDev* s
 // coordinates in registers, and forms their keys for every direction of the task (packed FMAs over point pairs,
 // the direction's pairs from shared memory); warp g then takes direction g's steps between the passes alone.
 // X is read twice per task whatever its number of directions, and no key is stored, so 16 directions are in flight
-// per SM at any n.  About 25 instructions per key over both passes.
+// per SM at any n.  Measured at n = 10,000, d = 10 (10,000 directions, 247 us): 43 instructions a key over both passes,
+// the shared-memory pipe at 53% of its wavefronts (two fifths of them the reductions), issue slots at 50% with the 16
+// warps an SM holds.
 template <int D>
 __global__ void __launch_bounds__(SX_NT, 2) k_select_x(const TaskDev* __restrict__ tasks,
                                                      const SlotDev* __restrict__ slots,

@@ -453,7 +453,8 @@ cudaError_t launch_debug_dirs(uint64_t seed, int q, int round0, int m, int d, fl
 // bit set are near ties and take the exact test.  The directions stay in shared memory; the points come 16 dims at
 // a time, the next 16 in flight in registers.
 // Measured at d = 50, n = 100,000, 100 queries of 100 directions: 9.28 ms per round with 4 x 4 scalar outputs per
-// thread, 5.11 ms with this tile, 2.78 ms with the points also split (hd_parts): 46% of the FMA peak.
+// thread, 5.11 ms with this tile, 2.78 ms with the points also split (hd_parts), 2.57 ms with rows' own bounds (own_z):
+// half of the FMA peak.
 constexpr int HD_NT = 128;
 constexpr int HD_TJ = HD_ROWS;   // rows (query, direction) per CTA
 constexpr int HD_PC = 256;       // points per chunk
