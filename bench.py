@@ -56,14 +56,17 @@ SM_MAX_MHZ_NOMINAL = 2070.0
 # valid only for the kernel source it was taken from: `src_sha16` is the SHA-256 prefix of those files at
 # capture time, and a mismatch (the kernel changed since) reports null.
 CAPTURED = {
-    # k_pdap2<2,12>, d = 10, n = 10,000, 50,000 directions per launch: rounds 10-12 of each kind (six launches
-    # of the first warm-up step): DRAM bytes and warp instructions per (point, direction) element, averaged
-    "k_pdap2_c2": {"src": ("paper_2506_08262_gb300/csrc/pdap.cu", "paper_2506_08262_gb300/csrc/rrs_internal.h"),
-                   "src_sha16": "8f7dbf26a8a98cf6", "traffic": 3.548e6, "warp_instr_per_element": 2.105},
+    # the headline's selection kernel, k_select_x<10>, d = 10, n = 10,000, 50,000 directions per launch: rounds 10-12
+    # of each kind (six launches of the first warm-up step): DRAM bytes and warp instructions per (point, direction)
+    # element, averaged
+    "k_pdap2_c2": {"src": ("paper_2506_08262_gb300/csrc/pdap_select.cu", "paper_2506_08262_gb300/csrc/pdap_common.cuh",
+                           "paper_2506_08262_gb300/csrc/packed_fma.cuh",
+                           "paper_2506_08262_gb300/csrc/rrs_internal.h"),
+                   "src_sha16": "fdc60efaa69a89fd", "traffic": 3.198e6, "warp_instr_per_element": 1.305},
     # k_hd_tc<256>, 10,000 queries x 100 directions x 100,000 points, d = 50: one launch
     "k_hd_tc_c3": {"src": ("paper_2506_08262_gb300/csrc/hd_tc.cu", "paper_2506_08262_gb300/csrc/async_sync.cuh",
                            "paper_2506_08262_gb300/csrc/rrs_device.cuh"),
-                   "src_sha16": "78f16dea39c9afd0", "traffic": 290.41e6},
+                   "src_sha16": "e66bab62d7e3c72f", "traffic": 289.92e6},
 }
 ISSUE_PER_SM_PER_CLK = 4     # one warp instruction per clock on each of the four SM sub-partitions
 
@@ -96,7 +99,7 @@ def parse():
     ap.add_argument("--cpu-full", action="store_true",
                     help="--impl reference: time the oracle on every query of the workload per step")
     ap.add_argument("--no-autotune", action="store_true",
-                    help="headline: keep the shared-memory heuristic for the selection kernel's directions per CTA")
+                    help="headline: keep the library's default selection kernel")
     ap.add_argument("--no-halfspace", action="store_true", help="skip the secondary d=50 halfspace measurement")
     ap.add_argument("--nq", type=int, default=0, help="queries (default: the full workload)")
     ap.add_argument("--workload", choices=["c1", "c2", "c3", "c4", "c5", "grid", "ranks", "convergence"], default="c2",
@@ -360,7 +363,7 @@ def run_ours(args):
     stream = torch.cuda.current_stream(dev)
     flush = torch.empty(L2_FLUSH_BYTES, dtype=torch.uint8, device=dev)
 
-    # the autotuner times each choice; --no-autotune keeps the library's shared-memory heuristic (used for
+    # the autotuner times each choice; --no-autotune keeps the library's default kernel (used for
     # profiler captures, where the probe timings are distorted by the profiler itself)
     tuned = ({workloads.KIND_NAMES[kd]: rrs.rrs_autotune(ctx, did, kd, k, r) for kd in kinds}
              if not args.no_autotune else "heuristic")
