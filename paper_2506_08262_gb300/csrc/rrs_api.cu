@@ -680,15 +680,15 @@ rrs_status rrs_register_dataset(rrs_ctx* ctx, const void* X, int64_t n, int32_t 
     const void* src = X;
     cudaStream_t st = 0;
     if (!x_on_device) {
-        CUDA_TRY(cudaMalloc(&staged, esz * n * d));
+        CUDA_TRY(ctx_malloc(ctx, &staged, esz * n * d));
         CUDA_TRY(cudaMemcpy(staged, X, esz * n * d, cudaMemcpyHostToDevice));
         src = staged;
     }
-    cudaError_t e = cudaMalloc(&D.X32, b32);
-    if (e == cudaSuccess && bt) e = cudaMalloc(&D.Xt, bt);
-    if (e == cudaSuccess && b64) e = cudaMalloc(&D.X64, b64);
-    if (e == cudaSuccess) e = cudaMalloc(&D.xnorm, bn);
-    if (e == cudaSuccess) e = cudaMalloc(&D.center, bmom);
+    cudaError_t e = ctx_malloc(ctx, &D.X32, b32);
+    if (e == cudaSuccess && bt) e = ctx_malloc(ctx, &D.Xt, bt);
+    if (e == cudaSuccess && b64) e = ctx_malloc(ctx, &D.X64, b64);
+    if (e == cudaSuccess) e = ctx_malloc(ctx, &D.xnorm, bn);
+    if (e == cudaSuccess) e = ctx_malloc(ctx, &D.center, bmom);
     if (e == cudaSuccess) e = cudaMemset(ctx->d_err, 0, sizeof(int));
     if (e == cudaSuccess) e = launch_convert_dataset(src, dtype, n, d, D.ldx, D.X32, D.X64, D.xnorm, ctx->d_err, st);
     if (e == cudaSuccess && D.Xt) {
@@ -753,7 +753,7 @@ rrs_status rrs::ensure_bf16_planes(rrs_ctx* ctx, Dataset& D)
     const int kp = (int)align_up(D.d + 2, 64);
     const size_t bytes = sizeof(uint16_t) * 2 * (size_t)kp * D.n;
     if (!budget_ok(ctx, bytes)) return fail(RRS_ERR_BUDGET, "BF16 planes need %zu bytes", bytes);
-    CUDA_TRY(cudaMalloc(&D.Xbf, bytes));
+    CUDA_TRY(ctx_malloc(ctx, &D.Xbf, bytes));
     CUDA_TRY(launch_build_bf16_planes(D.X32, D.n, D.d, D.ldx, kp, D.Xbf, 0));
     CUDA_TRY(cudaDeviceSynchronize());
     ctx->launches++;
@@ -974,7 +974,7 @@ rrs_status rrs_depth_batched(rrs_ctx* ctx, const rrs_request* reqs, int32_t n_re
     if (!budget_ok(ctx, bytes)) return fail(RRS_ERR_BUDGET, "batched workspace needs %zu bytes", bytes);
     rrs_ctx::GraphEntry G;
     G.key = key;
-    CUDA_TRY(cudaMalloc(&G.ws, bytes));
+    CUDA_TRY(ctx_malloc(ctx, &G.ws, bytes));
     G.ws_bytes = bytes;
     Carve C;
     C.base = (char*)G.ws;
@@ -1066,7 +1066,7 @@ rrs_status rrs_debug_round_depths(rrs_ctx* ctx, int64_t dataset_id, const void* 
     if (s != RRS_OK) return s;
     const size_t bytes = plan_bytes(ctx, P) + sizeof(int64_t) * n_queries + 512;
     void* ws = nullptr;
-    CUDA_TRY(cudaMalloc(&ws, bytes));
+    CUDA_TRY(ctx_malloc(ctx, &ws, bytes));
     Carve C;
     C.base = (char*)ws;
     carve_plan(P, C);

@@ -74,6 +74,17 @@ struct rrs_ctx {
 };
 
 namespace rrs {
+// cudaMalloc for what a context keeps; where memory is short, what its pool holds between calls goes back first.
+template <class T>
+cudaError_t ctx_malloc(rrs_ctx* ctx, T** p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc((void**)p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    cudaMemPoolTrimTo(ctx->pool, 0);
+    return cudaMalloc((void**)p, bytes);
+}
+
 // Build (once) the BF16 hi/lo planes the tensor-core halfspace kernel streams;
 // UNSUPPORTED for d + 2 > 128, BUDGET when they do not fit the context's budget.
 rrs_status ensure_bf16_planes(rrs_ctx* ctx, Dataset& D);

@@ -308,7 +308,7 @@ rrs_status rrs_server_create(rrs_ctx* ctx, int32_t max_slots, int32_t max_dirs_p
         delete S;
         return sfail(RRS_ERR_BUDGET, "server arena needs %zu bytes", off);
     }
-    cudaError_t e = cudaMalloc(&S->arena, off);
+    cudaError_t e = ctx_malloc(ctx, &S->arena, off);
     if (e != cudaSuccess) {
         cudaGetLastError();
         delete S;
