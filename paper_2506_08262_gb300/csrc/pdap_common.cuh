@@ -113,17 +113,18 @@ __device__ void gminmax(const Grp<GS>& q, float lo, float hi, CT& C, float& olo,
 {
     lo = warp_min(lo);
     hi = warp_max(hi);
+    constexpr int NW = GS / 32;
     if ((q.t & 31) == 0) {
         C.fred[q.g][q.t >> 5] = lo;
-        C.fred[q.g][NWARP + (q.t >> 5)] = hi;
+        C.fred[q.g][NW + (q.t >> 5)] = hi;
     }
     q.sync();
     olo = C.fred[q.g][0];
-    ohi = C.fred[q.g][NWARP];
+    ohi = C.fred[q.g][NW];
 #pragma unroll
-    for (int i = 1; i < GS / 32; ++i) {
+    for (int i = 1; i < NW; ++i) {
         olo = fminf(olo, C.fred[q.g][i]);
-        ohi = fmaxf(ohi, C.fred[q.g][NWARP + i]);
+        ohi = fmaxf(ohi, C.fred[q.g][NW + i]);
     }
     q.sync();
 }

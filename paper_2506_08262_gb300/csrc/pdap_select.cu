@@ -106,7 +106,7 @@ constexpr int RF_DONE = 0, RF_COUNT = 1, RF_LIST = 2, RF_TIES = 3, RF_PIVOT = 4,
 template <int NG>
 struct CtlS {
     int red[NG][NWARP / NG];
-    float fred[NG][2 * NWARP];
+    float fred[NG][2 * NWARP / NG];   // two per warp of a group
     int fill[NG][2];
     int f_b1[NG], f_c1[NG], f_b2[NG], f_c2[NG];
     float pv1[NG], pv2[NG];
@@ -115,6 +115,9 @@ struct CtlS {
     SelPar par[NG];
     SelRef rf[NG];
 };
+
+// two k_select_x CTAs, with the 1 KB that each reserves, fill the 228 KB of an SM at most
+static_assert(2 * (SX_SMEM + sizeof(CtlS<SX_G>) + 1024) <= 228 * 1024, "k_select_x: two CTAs per SM");
 
 __device__ __forceinline__ float lo_f(unsigned long long v) { return __uint_as_float((unsigned)v); }
 __device__ __forceinline__ float hi_f(unsigned long long v) { return __uint_as_float((unsigned)(v >> 32)); }
@@ -579,7 +582,7 @@ __device__ __forceinline__ void sel_rank(const Grp<GS>& q, const float* B, const
 {
     // a larger group ranks pairs side by side, and its walks end in barriers: n = 100,000, d = 100, runs of about 150
     // pairs and 128 threads, 60.2 against 61.4 ms
-    if (cnt <= (GS == 32 ? 128 : 512)) gpick(q, B, I, cnt, s1, s2, C, v1, v2, i1, i2);
+    if (cnt <= (GS == 32 ? 192 : 512)) gpick(q, B, I, cnt, s1, s2, C, v1, v2, i1, i2);
     else sel_bisect<GS, CT>(q, B, I, cnt, s1, s2, C, v1, v2, i1, i2);
 }
 
@@ -1588,15 +1591,21 @@ __global__ void __launch_bounds__(SX_NT, 2) k_select_x(const TaskDev* __restrict
     }
     __syncthreads();
 
+    // the runs' record: held in registers through the next pass where the coordinates leave room for it, else in shared
+    // memory (n = 10,000, d = 10: 22.4 against 24.9 ms with spills; a short pass feels the way there and back: n = 599,
+    // d = 4 10.5 against 10.7 ms)
+    constexpr bool HELD = D <= 6;
+    SelRuns held{};
     unsigned* H = area + w * words;
     if (w < GA) {
         sel_prefix(q, H, nb, C);
         SelLong X;
         const SelRuns R = sel_runs(H, nb, n, ap, par, X);
         if (R.fb && R.cnt0 > 0) par.dup = sel_twice(y, n);
-        if (lane == 0) {   // shared, not held in registers through the next pass
+        if (HELD) held = R;
+        if (lane == 0) {
             C.par[w] = par;
-            C.rf[w].R = R;
+            if (!HELD) C.rf[w].R = R;
             if (sel_long(R, nb)) C.rf[w].X = X;
         }
     }
@@ -1639,8 +1648,8 @@ __global__ void __launch_bounds__(SX_NT, 2) k_select_x(const TaskDev* __restrict
     ResDev* out = res + S.roff + T.j0 + w;
     bool more = false;
     if (w < GA) {
-        const SelRuns R = C.rf[w].R;
-        par = C.par[w];
+        const SelRuns R = HELD ? held : C.rf[w].R;
+        if (!HELD) par = C.par[w];
         const bool fast = !R.fb && (ap || R.second) && R.cnt <= 32 * FJ && R.cnt0 <= 32 && C.fill[w][0] == R.cnt &&
                           sel_picks_warp(R, par, H, nb, n, ap, out);
         more = !fast && !sel_picks<32, CtlS<SX_G>>(q, R, par, C, H, nb, n, ap, out);
