@@ -62,7 +62,7 @@ CAPTURED = {
     "k_pdap2_c2": {"src": ("paper_2506_08262_gb300/csrc/pdap_select.cu", "paper_2506_08262_gb300/csrc/pdap_common.cuh",
                            "paper_2506_08262_gb300/csrc/packed_fma.cuh",
                            "paper_2506_08262_gb300/csrc/rrs_internal.h"),
-                   "src_sha16": "fdc60efaa69a89fd", "traffic": 3.198e6, "warp_instr_per_element": 1.305},
+                   "src_sha16": "079abd8fdcc0c515", "traffic": 3.234e6, "warp_instr_per_element": 1.308},
     # k_hd_tc<256>, 10,000 queries x 100 directions x 100,000 points, d = 50: one launch
     "k_hd_tc_c3": {"src": ("paper_2506_08262_gb300/csrc/hd_tc.cu", "paper_2506_08262_gb300/csrc/async_sync.cuh",
                            "paper_2506_08262_gb300/csrc/rrs_device.cuh"),
